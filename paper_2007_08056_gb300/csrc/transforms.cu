@@ -1311,26 +1311,30 @@ cudaError_t launch_rowtile(const Problem& p, const Tables& t, int n_slices, cons
   a.zero64 = zero64;
   a.zero64_n = zero64_n;
   const size_t smem = rowtile_smem_bytes(p.K, kpad);
-  // the attribute and the occupancy are taken once per instance and device
-  // (kept per host thread)
-  thread_local size_t set_for[kMaxSlices + 1][16] = {};
-  thread_local int resident[kMaxSlices + 1][16] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 16) return cudaErrorInvalidDevice;
-  if (set_for[n_slices][dev] < smem) {
-    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // The shared-memory attribute belongs to the function, not to the host
+  // thread: every thread sets the same value, the most any row length needs,
+  // so that no thread lowers what another one relies on.
+  thread_local bool attr_set[kMaxSlices + 1][16] = {};
+  if (!attr_set[n_slices][dev]) {
+    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)rowtile_smem_bytes(kRowTileMaxK, kRowTileMaxK));
     if (e != cudaSuccess) return e;
-    set_for[n_slices][dev] = smem;
-    resident[n_slices][dev] = 0;
+    attr_set[n_slices][dev] = true;
   }
-  if (resident[n_slices][dev] == 0) {
+  // resident CTAs at this call's shared memory, kept for the size last asked
+  thread_local size_t resident_smem[kMaxSlices + 1][16] = {};
+  thread_local int resident[kMaxSlices + 1][16] = {};
+  if (resident_smem[n_slices][dev] != smem) {
     int sms = 0, per = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, RT_THREADS, smem);
     if (e != cudaSuccess) return e;
     resident[n_slices][dev] = sms * (per > 0 ? per : 1);
+    resident_smem[n_slices][dev] = smem;
   }
   const int64_t work = units[0] + units[1];
   const int64_t zero_ctas = (zero64_n + RT_THREADS - 1) / RT_THREADS;
@@ -1387,16 +1391,16 @@ cudaError_t launch_rowstream(const Problem& p, const Tables& t, int op, int n_sl
   if (nbuf > kRsMaxBufs) nbuf = kRsMaxBufs;
   if (nbuf < 2) return cudaErrorInvalidValue;
   const size_t smem = (size_t)nbuf * row_bytes;
-  // the attribute is set once per instance and device (kept per host thread)
-  thread_local size_t set_for[2][kMaxSlices + 1][16] = {};
+  // (the attribute belongs to the function: every thread sets the same value)
+  thread_local bool attr_set[2][kMaxSlices + 1][16] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 16) return cudaErrorInvalidDevice;
-  if (set_for[C > 1][n_slices][dev] < smem) {
-    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!attr_set[C > 1][n_slices][dev]) {
+    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsSmem);
     if (e != cudaSuccess) return e;
-    set_for[C > 1][n_slices][dev] = smem;
+    attr_set[C > 1][n_slices][dev] = true;
   }
   int sms = 0;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -55,3 +55,30 @@ def test_two_threads_two_streams(sc):
     for res in results:
         for prec, got in res:
             assert np.linalg.norm(got - want) <= tol[prec] * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("long_k,short_k", [((4, 16, 16), (2, 5, 3)), ((8, 32, 8), (8, 24, 2))],
+                         ids=["short_rows", "long_rows"])
+def test_shorter_rows_on_another_thread(sc, long_k, short_k):
+    """A kernel's shared-memory limit belongs to the function, not to a thread:
+    a second thread with shorter rows (autograd's backward thread, say) must not
+    lower it below what the first thread has already asked for."""
+    def run(dims):
+        G, virt, occ = dims
+        c = WL.cc_ladder(G, G * virt, G * occ)
+        gen = torch.Generator(device="cuda").manual_seed(1)
+        p = sc.Plan(c.einsum, c.moduli, spec(c.u), spec(c.v), "split_bf16")
+        x = [torch.randn(s, generator=gen, dtype=torch.float64, device="cuda") for s in (p.shape_u, p.shape_v)]
+        p.contract(*x)
+        torch.cuda.synchronize()
+        p.check_device_error()
+        return p.info.single_read_prep
+
+    def other():
+        torch.cuda.set_device(0)
+        return run(short_k)
+
+    kernels = run(long_k)
+    with ThreadPoolExecutor(max_workers=1) as ex:
+        assert ex.submit(other).result() & kernels   # the same preparation kernel
+    assert run(long_k) == kernels
