@@ -199,7 +199,8 @@ KERNEL_SOURCES = {
     "prep_kernel": ("transforms.cu", "symctr_internal.h"),
     "rowtile_kernel": ("transforms.cu", "symctr_internal.h"),
     "rowstream_kernel": ("transforms.cu", "symctr_internal.h"),
-    "gemm_tc_kernel": ("gemm_tc.cu", "symctr_internal.h"),
+    "gemm_tc_kernel": ("gemm_tc.cu", "tc_common.cuh", "symctr_internal.h"),
+    "gemm_tc10_kernel": ("gemm_tc10.cu", "tc_common.cuh", "symctr_internal.h"),
     "gemm_f64": ("gemm_f64.cu", "symctr_internal.h"),
 }
 
@@ -241,14 +242,22 @@ def peaks():
     return p
 
 
+def digit_planes(n_slices):
+    """16-bit planes per operand of the split form: four FP16 digits of 10 bits for
+    the default n_slices = 5, else n_slices BF16 digits of 8 bits.  Planes i and j
+    are multiplied where i + j is below their count."""
+    return 4 if n_slices == 5 else n_slices
+
+
 def prep_bytes(pl):
     """Algorithmic bytes of one operand-prep launch: every aligned operand
     element read once as float64 and written once in the GEMM's operand format
-    (S BF16 slices, or one TF32 word), plus one int32 exponent per row."""
+    (the split form's digit planes, or one TF32 word), plus one int32 exponent
+    per row."""
     i = pl.info
     elems = i.aligned_numel_u + i.aligned_numel_v
     if i.precision == 1:
-        return elems * (8 + 2 * i.n_slices) + 4 * i.n_q * (i.M + i.N)
+        return elems * (8 + 2 * digit_planes(i.n_slices)) + 4 * i.n_q * (i.M + i.N)
     return elems * (8 + 4)
 
 
@@ -280,9 +289,11 @@ def rooflines(args, plans, prep, gemm, pk):
     out = []
     gemm_ms = sum(gemm)
     if args.precision == "split_bf16":
-        pairs = [pl.info.n_slices * (pl.info.n_slices + 1) // 2 for pl in plans]
+        planes = [digit_planes(pl.info.n_slices) for pl in plans]
+        pairs = [n * (n + 1) // 2 for n in planes]
         work = sum(pl.useful_flops * k for pl, k in zip(plans, pairs))
-        kernel, bound, unit, peak = "gemm_tc_kernel", "tensor", "TFLOP/s", pk["bf16_tflops"]
+        kernel = "gemm_tc10_kernel" if plans[0].info.n_slices == 5 else "gemm_tc_kernel"
+        bound, unit, peak = "tensor", "TFLOP/s", pk["bf16_tflops"]
         peak_src = f"{pk['src']} bf16 burst"
     elif args.precision == "tf32":
         work = sum(pl.useful_flops for pl in plans)
@@ -458,7 +469,7 @@ def run_ours(args, rank, world):
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,
-        "dtype": {"split_bf16": "bf16 slices x5, fp32 accumulate, int64 combine, f64 out",
+        "dtype": {"split_bf16": "fp16 digits x4 (39-bit operands), fp32 accumulate, int64 combine, f64 out",
                   "tf32": "tf32, fp32 accumulate, f64 out", "fp64": "f64"}[args.precision],
         "data": "synthetic (seeded N(0,1) reduced forms)",
         "config": {"workload": name, "precision": args.precision,

@@ -101,7 +101,7 @@ typedef struct {
   int32_t moduli[SYMCTR_MAX_MODULI];
   int32_t group_order;          /* G = product of moduli */
   int32_t precision;            /* symctr_precision */
-  int32_t n_slices;             /* BF16 slices per operand (split form), else 0 */
+  int32_t n_slices;             /* split form: 8 n_slices - 1 bits per operand, else 0 */
   int8_t signs_w[SYMCTR_MAX_ORDER];
   int32_t charge_w[SYMCTR_MAX_MODULI];
   int64_t dims_w[SYMCTR_MAX_ORDER];
@@ -188,7 +188,8 @@ typedef struct {
  *  signs_w_or_null / charge_w_or_null : optional check of the output law; the
  *             derived law (c^U on free-U modes, -sigma c^V on free-V modes,
  *             Z_U - sigma Z_V) or its global negation is accepted.
- *  prec, n_slices : precision form; n_slices = 0 picks the default (5).
+ *  prec, n_slices : precision form; the split form keeps 8 n_slices - 1 bits of
+ *             an operand (below its row's scale); n_slices = 0 picks the default (5).
  * Returns SYMCTR_OK and *out, or an error status and *out = NULL.  Host only. */
 SYMCTR_API symctr_status symctr_plan_create(const char* einsum, int n_moduli, const int32_t* moduli,
                                  const int8_t* signs_u, const int32_t* charge_u,

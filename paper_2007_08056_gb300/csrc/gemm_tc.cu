@@ -3,7 +3,8 @@
 // tcgen05.ld epilogue that writes W's standard reduced form directly (the
 // output step of Alg. 2 fused into the epilogue).
 //
-// Split-BF16 form (Ozaki-style; the paper has no mixed-precision path).
+// Split-BF16 form (Ozaki-style; the paper has no mixed-precision path), here for
+// n_slices = 2, 3, 4 and 6; the default 5 runs gemm_tc10.cu.
 //   Operands arrive as S BF16 slices, slice i holding balanced digits
 //   a_i * 2^(-8i), |a_i| <= 128, plus one binary exponent per aligned row.
 //   Slice-pair products a_i b_j (|.| <= 2^14) are summed on the tensor core in
@@ -35,13 +36,9 @@
 // 512 TMEM columns allocated (4 x 128 FP32 accumulators in the split form).
 // Every wait is bounded: on expiry the kernel records DEVERR_TIMEOUT in the
 // workspace error word, drains its own copies and MMAs, frees TMEM, returns.
-#include <cuda.h>
-#include <cstdint>
 #include <cstdio>
-#include <type_traits>
-#include <utility>
 
-#include "symctr_internal.h"
+#include "tc_common.cuh"
 
 namespace symctr {
 
@@ -50,7 +47,6 @@ namespace {
 constexpr int TM = 128;
 constexpr int NTHREADS = 384;
 constexpr int EPI_WARP0 = 4;
-constexpr int kExpBias = 4096;     // row exponents are stored biased (0 = all-zero row)
 // Every kFoldChunks exact drains, the rounded accumulator of diagonals >= 3 is
 // folded as well: its part in units of 2^-16 moves into the int32 running sum
 // of diagonal 2 and only the remainder (|r| <= 2^-17) stays in TMEM, so the
@@ -64,8 +60,6 @@ constexpr int kFoldChunks = 16;
 __host__ __device__ constexpr uint32_t drained_after(int c) {
   return c < 0 ? 7u : (4u | (((c + 1) % 2 == 0) ? 2u : 0u) | (((c + 1) % 4 == 0) ? 1u : 0u));
 }
-constexpr long long kTimeoutCycles = 4000000000ll;  // ~2 s per wait at 2 GHz
-
 enum Mode { MODE_SPLIT = 0, MODE_TF32 = 1 };
 
 // Tile shapes per form: the split form 128 x 128 (four accumulators fill
@@ -85,163 +79,6 @@ struct TileCfg {
   static constexpr int LD = N + 1;                           // staging row stride (elements)
   static constexpr size_t EPI_BYTES = (size_t)TM * LD * (KIND == MODE_SPLIT ? 8 : 4);
 };
-
-// ---------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ uint32_t su32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(su32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(su32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(su32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-struct Ctl {
-  volatile int abort;
-  unsigned* err;
-};
-
-// Bounded wait: true when the phase completed; false on timeout or abort.
-// The budget is counted in SM clock cycles (clock64 is cheap to read; about
-// 2 s at the maximum SM clock, longer at lower clocks).
-__device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity, Ctl* ctl,
-                                           long long limit = kTimeoutCycles) {
-  if (mbar_test(bar, parity)) return true;
-  const long long t0 = clock64();
-  for (;;) {
-    if (mbar_test(bar, parity)) return true;
-    if (ctl->abort) return false;
-    if (clock64() - t0 > limit) {
-      atomicOr(ctl->err, (unsigned)DEVERR_TIMEOUT);
-      ctl->abort = 1;
-      return false;
-    }
-  }
-}
-
-// Same, for threads with nothing else to do: the hardware suspends them
-// between polls (suspend-time hint), so they do not take issue slots from
-// the producer and MMA threads.
-__device__ __forceinline__ bool mbar_test_sleep(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(su32(bar)), "r"(parity), "r"(1000000u)
-      : "memory");
-  return ok != 0;
-}
-
-__device__ __forceinline__ bool wait_phase_sleep(uint64_t* bar, uint32_t parity, Ctl* ctl) {
-  const long long t0 = clock64();
-  for (;;) {
-    if (mbar_test_sleep(bar, parity)) return true;
-    if (ctl->abort) return false;
-    if (clock64() - t0 > kTimeoutCycles) {
-      atomicOr(ctl->err, (unsigned)DEVERR_TIMEOUT);
-      ctl->abort = 1;
-      return false;
-    }
-  }
-}
-
-__device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, uint64_t* bar, void* dst,
-                                            int c0, int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(su32(dst)),
-      "l"(map), "r"(su32(bar)), "r"(c0), "r"(c1), "r"(c2)
-      : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   su32(bar))
-               : "memory");
-}
-// 4 consecutive 32-bit TMEM columns of this warp's 32 lanes.
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(taddr));
-}
-
-// 16 consecutive 32-bit TMEM columns of this warp's 32 lanes.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-// 8 consecutive 32-bit TMEM columns of this warp's 32 lanes.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                 "=r"(r[7])
-               : "r"(taddr));
-}
-template <int W>
-__device__ __forceinline__ void tmem_ld_w(uint32_t taddr, uint32_t* r) {
-  if constexpr (W == 16) tmem_ld16(taddr, r);
-  else if constexpr (W == 8) tmem_ld8(taddr, r);
-  else tmem_ld4(taddr, r);
-}
-// Zeros into W consecutive 32-bit TMEM columns of this warp's 32 lanes.
-template <int W>
-__device__ __forceinline__ void tmem_zero_w(uint32_t taddr) {
-  const uint32_t z = 0u;
-  if constexpr (W == 16) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
-        "r"(z)
-        : "memory");
-  } else {
-    static_assert(W == 8, "8 or 16 columns");
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
-                 "r"(z)
-                 : "memory");
-  }
-}
-__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t* r) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr),
-               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
-               : "memory");
-}
-__device__ __forceinline__ void tmem_wait_st() {
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 
 // Shared-memory matrix descriptor: K-major, rows of ROW_BYTES swizzled over
 // their width (SWIZZLE_64B for 64-byte rows, SWIZZLE_128B for 128-byte rows),
@@ -266,176 +103,10 @@ __host__ __device__ constexpr uint32_t idesc() {
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
-// RN(R * 2^e) as float64 using integer operations only (ties to even).
-// Fast path: |R| < 2^53 and a normal result need no rounding, only a shift.
-__device__ __forceinline__ double i64_scaled_slow(long long Rv, int e) {
-  uint64_t sgn = Rv < 0 ? (1ull << 63) : 0ull;
-  uint64_t m = Rv < 0 ? (uint64_t)(-Rv) : (uint64_t)Rv;
-  int nb = 64 - __clzll((long long)m);
-  int be = e + nb - 1 + 1023;  // biased exponent of the leading bit
-  if (be >= 2047) return __longlong_as_double((long long)(sgn | 0x7FF0000000000000ull));
-  if (be <= 0) {
-    // subnormal: value / 2^-1074 = m * 2^(e + 1074)
-    int k = -(e + 1074);
-    uint64_t q;
-    if (k <= 0) {
-      q = m << (-k);
-    } else if (k >= 64) {
-      q = 0;
-      if (k == 64 && m > (1ull << 63)) q = 1;
-    } else {
-      q = m >> k;
-      uint64_t rem = m & ((1ull << k) - 1), half = 1ull << (k - 1);
-      if (rem > half || (rem == half && (q & 1))) ++q;
-    }
-    return __longlong_as_double((long long)(sgn | q));
-  }
-  int shift = nb - 53;
-  uint64_t q;
-  if (shift > 0) {
-    q = m >> shift;
-    uint64_t rem = m & ((1ull << shift) - 1), half = 1ull << (shift - 1);
-    if (rem > half || (rem == half && (q & 1))) ++q;
-    if (q == (1ull << 53)) {
-      q >>= 1;
-      ++be;
-      if (be >= 2047) return __longlong_as_double((long long)(sgn | 0x7FF0000000000000ull));
-    }
-  } else {
-    q = m << (-shift);
-  }
-  return __longlong_as_double((long long)(sgn | ((uint64_t)be << 52) | (q & ((1ull << 52) - 1))));
-}
-
-__device__ __forceinline__ double i64_scaled(long long Rv, int e) {
-  if (Rv == 0) return 0.0;
-  const uint64_t m = Rv < 0 ? (uint64_t)(-Rv) : (uint64_t)Rv;
-  if (m < (1ull << 53)) {
-    const int nb = 64 - __clzll((long long)m);
-    const int be = e + nb - 1 + 1023;
-    if (be > 0 && be < 2047) {
-      const uint64_t q = m << (53 - nb);
-      const uint64_t sgn = Rv < 0 ? (1ull << 63) : 0ull;
-      return __longlong_as_double((long long)(sgn | ((uint64_t)be << 52) | (q & ((1ull << 52) - 1))));
-    }
-  }
-  return i64_scaled_slow(Rv, e);
-}
-
-// Out-of-line copies for the rare entries of a batch (keeps the batch code small).
-__device__ __noinline__ double i64_scaled_rare(long long Rv, int e) { return i64_scaled_slow(Rv, e); }
-
-// The common case of i64_scaled without branches (selects only), so that a
-// batch of conversions interleaves: exact for Rv = 0, or |Rv| < 2^53 with a
-// normal result; `slow` is set for every other Rv.
-__device__ __forceinline__ double i64_scaled_common(long long Rv, int e, bool& slow) {
-  const uint64_t sm = (uint64_t)(Rv >> 63);   // all ones for Rv < 0
-  const uint64_t m = ((uint64_t)Rv ^ sm) - sm;
-  const int nb = 64 - __clzll((long long)m);
-  const int be = e + nb - 1 + 1023;
-  const uint64_t q = m << ((53 - nb) & 63);
-  const uint64_t bits = (sm << 63) | ((uint64_t)(unsigned)be << 52) | (q & ((1ull << 52) - 1));
-  slow = Rv != 0 && ((m >> 53) != 0 || (unsigned)(be - 1) >= 2046u);
-  return Rv == 0 ? 0.0 : __longlong_as_double((long long)bits);
-}
-
-// RN(Rv[j] * 2^e[j]) for a batch: the common case for all, the general routine
-// only for the entries that need it.
-template <int B>
-__device__ __forceinline__ void i64_scaled_batch(const long long (&Rv)[B], const int (&e)[B], double (&d)[B]) {
-  unsigned slow_mask = 0;
-#pragma unroll
-  for (int j = 0; j < B; ++j) {
-    bool sl;
-    d[j] = i64_scaled_common(Rv[j], e[j], sl);
-    slow_mask |= (unsigned)sl << j;
-  }
-  if (slow_mask) {
-#pragma unroll
-    for (int j = 0; j < B; ++j)
-      if ((slow_mask >> j) & 1u) d[j] = i64_scaled_rare(Rv[j], e[j]);
-  }
-}
-
-// Fire-and-forget 64-bit integer add in L2 (no value returned).
-__device__ __forceinline__ void red_add_u64(unsigned long long* a, unsigned long long v) {
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
-}
-
-// Exact float32 -> float64 with integer operations.
-__device__ __forceinline__ double f32_to_f64(uint32_t u) {
-  uint64_t sgn = (uint64_t)(u >> 31) << 63;
-  uint32_t e = (u >> 23) & 0xFF, m = u & 0x7FFFFF;
-  if (e == 0) {
-    if (m == 0) return __longlong_as_double((long long)sgn);
-    double v = i64_scaled((long long)m, -149);
-    return sgn ? -v : v;
-  }
-  if (e == 255) return __longlong_as_double((long long)(sgn | 0x7FF0000000000000ull | ((uint64_t)m << 29)));
-  return __longlong_as_double((long long)(sgn | ((uint64_t)(e - 127 + 1023) << 52) | ((uint64_t)m << 29)));
-}
-
-__device__ __noinline__ double f32_to_f64_rare(uint32_t u) { return f32_to_f64(u); }
-
-// f32_to_f64 for a batch: normal numbers and zeros without branches, the
-// general routine for subnormals, infinities and NaNs.
-template <int B>
-__device__ __forceinline__ void f32_to_f64_batch(const uint32_t (&u)[B], double (&d)[B]) {
-  unsigned slow_mask = 0;
-#pragma unroll
-  for (int j = 0; j < B; ++j) {
-    const uint32_t e = (u[j] >> 23) & 0xFFu;
-    const uint64_t sgn = (uint64_t)(u[j] >> 31) << 63;
-    const uint64_t bits = sgn | ((uint64_t)(e + 896u) << 52) | ((uint64_t)(u[j] & 0x7FFFFFu) << 29);
-    const bool zero = (u[j] << 1) == 0;
-    slow_mask |= (unsigned)(!zero && (e == 0 || e == 255)) << j;
-    d[j] = __longlong_as_double((long long)(zero ? sgn : bits));
-  }
-  if (slow_mask) {
-#pragma unroll
-    for (int j = 0; j < B; ++j)
-      if ((slow_mask >> j) & 1u) d[j] = f32_to_f64_rare(u[j]);
-  }
-}
-
-// Map-back stores of a batch of results of one column (rows m_first, + rstep,
-// ...): plain stores, or (complex products) adds, with the problem's sign; the
-// output mode is uniform, so the plain path loads nothing from W.
-// Rows or columns with offset -1 (general plans: absent from W) are not stored.
-template <int B, bool GEN>
-__device__ __forceinline__ void store_batch(const Problem& p, double* w, const int64_t (&ro)[B],
-                                            int64_t co, const double (&d)[B], int64_t m_first,
-                                            int rstep) {
-  if (co < 0) return;
-  if constexpr (!GEN) {
-#pragma unroll
-    for (int j = 0; j < B; ++j)
-      if (m_first + rstep * j < p.M && ro[j] >= 0) w[ro[j] + co] = d[j];
-  } else if (!p.accumulate) {
-#pragma unroll
-    for (int j = 0; j < B; ++j)
-      if (m_first + rstep * j < p.M && ro[j] >= 0) w[(int64_t)p.es * (ro[j] + co)] = signed_result(p, d[j]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < B; ++j)
-      if (m_first + rstep * j < p.M && ro[j] >= 0) w[(int64_t)p.es * (ro[j] + co)] += signed_result(p, d[j]);
-  }
-}
-
 // Descriptor offset of slice tile `i`, K step `kk` (16-byte units).
 template <int KIND>
 __host__ __device__ constexpr uint64_t dofs(int i, int kk) {
   return (uint64_t)((i * TM * TileCfg<KIND>::ROW_BYTES + kk * 32) >> 4);
-}
-
-// Compile-time loop: f(std::integral_constant<int, 0>) ... f(..<N-1>).
-template <typename F, int... Is>
-__device__ __forceinline__ void static_for_impl(F&& f, std::integer_sequence<int, Is...>) {
-  (f(std::integral_constant<int, Is>{}), ...);
-}
-template <int N, typename F>
-__device__ __forceinline__ void static_for(F&& f) {
-  static_for_impl(f, std::make_integer_sequence<int, N>{});
 }
 
 // One MMA on slice tiles (I, J) at K step KK: the descriptor offsets are
@@ -663,10 +334,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         uint8_t* sa = tiles + (size_t)st * stage_bytes;
         uint8_t* sb = sa + S * Cfg::A_BYTES;
         int kc = (kb0 + kb) * (Cfg::ROW_BYTES / args.ebytes);
-        for (int i = 0; i < S; ++i) {
-          tma_load_3d(&tma_a, &full[st], sa + i * Cfg::A_BYTES, kc, (int)m0, i * p.n_q + b);
-          tma_load_3d(&tma_b, &full[st], sb + i * Cfg::B_BYTES, kc, (int)n0, i * p.n_q + b);
-        }
+        // all S slice tiles of an operand in one copy
+        tma_load_4d(&tma_a, &full[st], sa, kc, (int)m0, b);
+        tma_load_4d(&tma_b, &full[st], sb, kc, (int)n0, b);
         ++issued;
       }
       if (ctl->abort) {
@@ -1042,19 +712,35 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-bool encode_map(CUtensorMap* map, const void* base, bool is_f32, int64_t kpad, int64_t rows,
-                int64_t planes, int box_rows);
+bool encode_map(CUtensorMap* map, const void* base, CUtensorMapDataType type, int64_t kpad, int64_t rows,
+                int64_t batches, int64_t planes, int box_k, int box_rows, int box_planes) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const int eb = type == CU_TENSOR_MAP_DATA_TYPE_FLOAT32 ? 4 : 2;
+  cuuint64_t dims[4] = {(cuuint64_t)kpad, (cuuint64_t)rows, (cuuint64_t)batches, (cuuint64_t)planes};
+  cuuint64_t strides[3] = {(cuuint64_t)(kpad * eb), (cuuint64_t)(kpad * eb * rows),
+                           (cuuint64_t)(kpad * eb * rows * batches)};
+  cuuint32_t box[4] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, 1, (cuuint32_t)box_planes};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = fn(map, type, 4, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  box_k * eb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
 
-// 3-D map over [planes][rows][kpad] with a (64-byte, box_rows, 1) box.  The
-// encoding is a pure function of its arguments, so the last few are kept per
-// host thread (a contraction called again on the same workspace reuses them).
-bool make_map(CUtensorMap* map, const void* base, bool is_f32, int64_t kpad, int64_t rows,
-              int64_t planes, int box_rows) {
+}  // namespace
+
+// The encoding is a pure function of its arguments, so the last few are kept
+// per host thread (a contraction called again on the same workspace reuses
+// them).
+bool make_map(CUtensorMap* map, const void* base, CUtensorMapDataType type, int64_t kpad, int64_t rows,
+              int64_t batches, int64_t planes, int box_k, int box_rows, int box_planes) {
   struct Entry {
     const void* base;
-    bool f32;
-    int64_t kpad, rows, planes;
-    int box_rows;
+    CUtensorMapDataType type;
+    int64_t kpad, rows, batches, planes;
+    int box_k, box_rows, box_planes;
     CUtensorMap map;
   };
   constexpr int kEntries = 8;
@@ -1062,37 +748,44 @@ bool make_map(CUtensorMap* map, const void* base, bool is_f32, int64_t kpad, int
   thread_local int used = 0, next = 0;
   for (int i = 0; i < used; ++i) {
     const Entry& e = cache[i];
-    if (e.base == base && e.f32 == is_f32 && e.kpad == kpad && e.rows == rows && e.planes == planes &&
-        e.box_rows == box_rows) {
+    if (e.base == base && e.type == type && e.kpad == kpad && e.rows == rows && e.batches == batches &&
+        e.planes == planes && e.box_k == box_k && e.box_rows == box_rows && e.box_planes == box_planes) {
       *map = e.map;
       return true;
     }
   }
-  if (!encode_map(map, base, is_f32, kpad, rows, planes, box_rows)) return false;
-  cache[next] = Entry{base, is_f32, kpad, rows, planes, box_rows, *map};
+  if (!encode_map(map, base, type, kpad, rows, batches, planes, box_k, box_rows, box_planes)) return false;
+  cache[next] = Entry{base, type, kpad, rows, batches, planes, box_k, box_rows, box_planes, *map};
   next = (next + 1) % kEntries;
   if (used < kEntries) ++used;
   return true;
 }
 
-bool encode_map(CUtensorMap* map, const void* base, bool is_f32, int64_t kpad, int64_t rows,
-                int64_t planes, int box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  int eb = is_f32 ? 4 : 2;
-  cuuint64_t dims[3] = {(cuuint64_t)kpad, (cuuint64_t)rows, (cuuint64_t)planes};
-  cuuint64_t strides[2] = {(cuuint64_t)(kpad * eb), (cuuint64_t)(kpad * eb * rows)};
-  // 128-byte rows with SWIZZLE_128B (TF32), 64-byte rows with SWIZZLE_64B (split)
-  const int rb = is_f32 ? TileCfg<MODE_TF32>::ROW_BYTES : TileCfg<MODE_SPLIT>::ROW_BYTES;
-  cuuint32_t box[3] = {(cuuint32_t)(rb / eb), (cuuint32_t)box_rows, 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = fn(map, is_f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
-                  const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  rb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
+cudaError_t launch_splitk_round(const Problem& p, const unsigned long long* wacc, const int32_t* eu,
+                                const int32_t* ev, const int64_t* wrow, const int64_t* wcol, double* w,
+                                const unsigned* err, cudaStream_t st) {
+  // one thread per kRoundRows outputs
+  const int64_t work = (int64_t)p.n_q * ((p.M + kRoundRows - 1) / kRoundRows) * p.N;
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t blocks = (work + kRoundThreads - 1) / kRoundThreads;
+  cudaLaunchConfig_t rc = {};
+  rc.gridDim = dim3((unsigned)(blocks < (int64_t)sms * 8 ? blocks : (int64_t)sms * 8));
+  rc.blockDim = dim3(kRoundThreads);
+  rc.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  rc.attrs = attr;
+  rc.numAttrs = 1;
+  const bool plain = p.es == 1 && !p.negate && !p.accumulate;
+  cudaError_t e = cudaLaunchKernelEx(&rc, plain ? splitk_round_kernel<false> : splitk_round_kernel<true>, p, wacc,
+                                     eu, ev, wrow, wcol, w, err);
+  ++g_kernel_launches;
+  return e;
 }
+
+namespace {
 
 template <int KIND, int S, int STAGES, bool GEN>
 cudaError_t launch_tc_mode(const Problem& p, const Tables& tab, const void* a, const void* bop, const int32_t* eu,
@@ -1100,8 +793,10 @@ cudaError_t launch_tc_mode(const Problem& p, const Tables& tab, const void* a, c
                       unsigned long long* wacc, cudaStream_t st) {
   const bool f32 = KIND == MODE_TF32;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, a, f32, kpad, p.M, (int64_t)S * p.n_q, TM) ||
-      !make_map(&mb, bop, f32, kpad, p.N, (int64_t)S * p.n_q, TileCfg<KIND>::N))
+  const CUtensorMapDataType type = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  const int box_k = TileCfg<KIND>::ROW_BYTES / (f32 ? 4 : 2);
+  if (!make_map(&ma, a, type, kpad, p.M, p.n_q, S, box_k, TM, S) ||
+      !make_map(&mb, bop, type, kpad, p.N, p.n_q, S, box_k, TileCfg<KIND>::N, S))
     return cudaErrorInvalidValue;
   TcArgs args;
   args.p = p;
@@ -1148,19 +843,7 @@ cudaError_t launch_tc_mode(const Problem& p, const Tables& tab, const void* a, c
   cudaError_t le = cudaLaunchKernelEx(&cfg, kern, ma, mb, args);
   ++g_kernel_launches;
   if (le != cudaSuccess || KIND != MODE_SPLIT || args.ksplit == 1) return le;
-  // the rounding of the split-K sums, one thread per kRoundRows outputs
-  const int64_t work = (int64_t)p.n_q * ((p.M + kRoundRows - 1) / kRoundRows) * p.N;
-  int sms = 148;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t blocks = (work + kRoundThreads - 1) / kRoundThreads;
-  cudaLaunchConfig_t rc = cfg;
-  rc.gridDim = dim3((unsigned)(blocks < (int64_t)sms * 8 ? blocks : (int64_t)sms * 8));
-  rc.blockDim = dim3(kRoundThreads);
-  rc.dynamicSmemBytes = 0;
-  le = cudaLaunchKernelEx(&rc, splitk_round_kernel<GEN>, p, (const unsigned long long*)wacc, eu, ev,
-                          tab.wrow, tab.wcol, w, (const unsigned*)err);
-  ++g_kernel_launches;
-  return le;
+  return launch_splitk_round(p, wacc, eu, ev, tab.wrow, tab.wcol, w, err, st);
 }
 
 template <int KIND, int S, int STAGES>
@@ -1184,7 +867,7 @@ cudaError_t launch_gemm_split(const Problem& p, const Tables& tab, int n_slices,
     case 2: return launch_tc<MODE_SPLIT, 2, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
     case 3: return launch_tc<MODE_SPLIT, 3, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
     case 4: return launch_tc<MODE_SPLIT, 4, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
-    case 5: return launch_tc<MODE_SPLIT, 5, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
+    case 5: return launch_gemm_split10(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
     case 6: return launch_tc<MODE_SPLIT, 6, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
   }
   return cudaErrorInvalidValue;

@@ -75,8 +75,8 @@ Layout make_layout(const Problem& pr, bool tensor_core, bool general, symctr_pre
       return L;
     }
     if (prec == SYMCTR_SPLIT_BF16) {
-      L.off_a = region(ra * 2 * n_slices);
-      L.off_b = region(rb * 2 * n_slices);
+      L.off_a = region(ra * 2 * digit_planes(n_slices));
+      L.off_b = region(rb * 2 * digit_planes(n_slices));
       L.off_ea = region(nq * pr.M * 4);
       L.off_eb = region(nq * pr.N * 4);
       if (prep_partials_entries(pr) > 0) L.off_part = region(prep_partials_entries(pr) * 4);

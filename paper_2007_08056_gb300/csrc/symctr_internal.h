@@ -258,6 +258,10 @@ enum : unsigned { DEVERR_NONE = 0, DEVERR_TIMEOUT = 1, DEVERR_NONFINITE = 2 };
 // Split-precision constants.
 constexpr int kSliceBits = 8;       // bits per balanced BF16 digit
 constexpr int kMaxSlices = 6;
+// Planes of 16-bit digits per operand: the default split (n_slices = 5, 39 bits
+// and a sign) holds four FP16 digits of 10 bits, the others n_slices BF16
+// digits of 8 bits.
+inline int digit_planes(int n_slices) { return n_slices == 5 ? 4 : n_slices; }
 constexpr int kKBlock = 32;         // K per pipeline stage (64-byte rows of BF16)
 constexpr int kKChunk = 64;         // K between exact flushes of the top accumulators
 
@@ -306,6 +310,10 @@ cudaError_t launch_gemm_split(const Problem& p, const Tables& t, int n_slices, c
                               const uint16_t* vs, const int32_t* eu, const int32_t* ev,
                               int64_t kpad, double* w, unsigned* err, int ksplit,
                               unsigned long long* wacc, cudaStream_t st);
+cudaError_t launch_gemm_split10(const Problem& p, const Tables& t, const uint16_t* us, const uint16_t* vs,
+                                const int32_t* eu, const int32_t* ev, int64_t kpad, double* w,
+                                unsigned* err, int ksplit, unsigned long long* wacc,
+                                cudaStream_t st);
 cudaError_t launch_gemm_tf32(const Problem& p, const Tables& t, const float* u, const float* v,
                              int64_t kpad, double* w, unsigned* err, cudaStream_t st);
 

@@ -10,6 +10,7 @@
 #include <cstdint>
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "symctr_internal.h"
 
@@ -392,12 +393,58 @@ __device__ __forceinline__ void put_digits(uint64_t y0, uint64_t y1, uint32_t* d
   }
 }
 
+// ---- default split (S = 5): the same 39-bit X as four FP16 digits ----
+// Balanced base-1024 digits a_0..a_3 (a_0 on top), |a_i| <= 512, each stored as
+// an FP16 integer (exact).  With B = 512 (1024^3 + 1024^2 + 1024 + 1), the word
+// Y = 4 (X + B) + 2 bits of fraction holds a_3 + 512, a_2 + 512, a_1 + 512 in
+// bits 2, 12, 22 and a_0 + 512 (up to 1024) from bit 32.
+constexpr uint64_t kBias10 = 512ull * ((1ull << 30) + (1ull << 20) + (1ull << 10) + 1ull);
+
+// Y for rows whose k0 >= 66 (every scale above 2^-971), rounded half up: the
+// mantissa's one's complement for negative entries, one arithmetic shift that
+// keeps two fraction bits, one add of 4 B + 2.  (An entry below the normal
+// range shifts out altogether at these scales, so its implicit bit is moot;
+// the one's complement is off by 2^-14 of X's unit at most, before rounding.)
+__device__ __forceinline__ uint64_t y10_fast(double x, int k0) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t sgn = (uint32_t)((int32_t)hi >> 31);
+  const uint32_t mh = ((hi & 0xFFFFFu) | 0x100000u) ^ sgn, ml = lo ^ sgn;
+  const int k = min(k0 - 2 - (int)((hi >> 20) & 0x7FFu), 63);
+  const int64_t v = (int64_t)(((uint64_t)mh << 32) | ml) >> k;
+  return (uint64_t)v + (4 * kBias10 + 2);
+}
+__device__ __forceinline__ uint64_t y10(double x, int k0) {
+  return ((uint64_t)fixed_point(x, k0) + kBias10) << 2;
+}
+
+// The digits of two entries as packed FP16: u in [0, 1024] under the exponent
+// of 1024 is the FP16 1024 + u, and subtracting 1536 leaves u - 512 (exact).
+__device__ __forceinline__ uint32_t digit10(uint32_t w) {
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), __half2half2(__ushort_as_half(0x6600)));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ void digits10(uint64_t ya, uint64_t yb, uint32_t (&d)[4]) {
+  const uint32_t la = (uint32_t)ya, lb = (uint32_t)yb, m = 0x03FF03FFu, one = 0x64006400u;
+  d[0] = digit10(__byte_perm((uint32_t)(ya >> 32), (uint32_t)(yb >> 32), 0x5410) + one);
+  d[1] = digit10(((__byte_perm(la, lb, 0x7632) >> 6) & m) | one);
+  d[2] = digit10(((__byte_perm(la, lb, 0x6521) >> 4) & m) | one);
+  d[3] = digit10(((__byte_perm(la, lb, 0x5410) >> 2) & m) | one);
+}
+
 template <int S>
 __device__ __forceinline__ void put_slices_pair(double x0, double x1, int k0, uint32_t* dst,
                                                 int64_t stride) {
-  const uint64_t y0 = (uint64_t)(fixed_point(x0, k0) + (int64_t)digit_bias(S));
-  const uint64_t y1 = (uint64_t)(fixed_point(x1, k0) + (int64_t)digit_bias(S));
-  put_digits<S>(y0, y1, dst, stride);
+  if constexpr (S == 5) {
+    uint32_t d[4];
+    if (k0 >= 66) digits10(y10_fast(x0, k0), y10_fast(x1, k0), d);
+    else digits10(y10(x0, k0), y10(x1, k0), d);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dst[(int64_t)i * stride] = d[i];
+  } else {
+    const uint64_t y0 = (uint64_t)(fixed_point(x0, k0) + (int64_t)digit_bias(S));
+    const uint64_t y1 = (uint64_t)(fixed_point(x1, k0) + (int64_t)digit_bias(S));
+    put_digits<S>(y0, y1, dst, stride);
+  }
 }
 
 // Four adjacent columns of one row: per slice, four BF16 digits in one 8-byte
@@ -416,9 +463,24 @@ __device__ __forceinline__ void put_digits_quad(const uint64_t (&y)[4], uint2* d
 template <int S>
 __device__ __forceinline__ void put_slices_quad(const double (&x)[4], int k0, uint2* dst, int64_t stride) {
   uint64_t y[4];
+  if constexpr (S == 5) {
+    if (k0 >= 66) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) y[j] = (uint64_t)(fixed_point(x[j], k0) + (int64_t)digit_bias(S));
-  put_digits_quad<S>(y, dst, stride);
+      for (int j = 0; j < 4; ++j) y[j] = y10_fast(x[j], k0);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) y[j] = y10(x[j], k0);
+    }
+    uint32_t a[4], b[4];
+    digits10(y[0], y[1], a);
+    digits10(y[2], y[3], b);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dst[(int64_t)i * stride] = make_uint2(a[i], b[i]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = (uint64_t)(fixed_point(x[j], k0) + (int64_t)digit_bias(S));
+    put_digits_quad<S>(y, dst, stride);
+  }
 }
 
 __device__ __forceinline__ float tf32_round(double x) {
@@ -1273,8 +1335,8 @@ size_t rowtile_smem_bytes(int64_t K, int64_t kpad) {
 
 cudaError_t launch_rowtile(const Problem& p, const Tables& t, int n_slices, const bool* on,
                            const double* u, const double* v, void* ua, void* va, int32_t* eu,
-                           int32_t* ev, int64_t kpad, unsigned* err, unsigned long long* zero64,
-                           int64_t zero64_n, cudaStream_t st) {
+                           int32_t* ev, int64_t kpad, unsigned* err,
+                           unsigned long long* zero64, int64_t zero64_n, cudaStream_t st) {
   if (n_slices < 1 || n_slices > kMaxSlices || p.es != 1 || p.K < 1 || kpad > kRowTileMaxK ||
       kpad % 32 != 0 || kpad < p.K)
     return cudaErrorInvalidValue;

@@ -1,0 +1,70 @@
+"""The default split form (four FP16 digits of 10 bits) at the sizes and values
+where its GEMM can go wrong: half tiles and remainders of M and N, one column of
+K up to several folds of the diagonals, split K ranges, and entries whose digits
+are at their limits so that every partial sum is.
+
+An entry is rounded to 39 bits below its row's 2^(E+1) and the digit pairs with
+i + j >= 4 are dropped (three of 2^-40 each), so an output is within
+K 2^(Eu+1) 2^(Ev+1) (2 x 2^-40 + 3 x 2^-40) of the exact sum, plus the rounding
+of the diagonals d >= 2 (2^-20 of the products, FP32 sums of at most 512 columns
+between folds: below 2^-38 K of the same scale) and of R (2^-39); 2^-36 K covers
+them all."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(8, 8, 1), (127, 63, 31), (128, 64, 33), (129, 65, 64), (257, 127, 96), (40, 129, 577),
+         (8, 200, 1100), (9, 8, 8200), (130, 140, 32768)]
+
+
+@pytest.fixture(scope="module")
+def sc():
+    if not torch.cuda.is_available():
+        pytest.fail("a GPU test ran without a visible GPU")
+    import paper_2007_08056_gb300 as mod
+    mod.load()
+    return mod
+
+
+def draw(kind, shape, rng):
+    if kind == "normal":
+        return rng.standard_normal(shape) * 2.0 ** rng.integers(-30, 30, shape[:-1] + (1,))
+    if kind == "largest":      # rounds up to the next power of two: top digits of 512
+        return np.full(shape, 2.0 - 2.0 ** -45)
+    if kind == "aligned":      # every digit 410 in size: all partial sums grow with K
+        return np.full(shape, 0.1) * np.where(rng.random(shape[:-1] + (1,)) < 0.5, 1.0, -1.0)
+    # lower digits of -512: X = 300 2^30 - 512 (2^20 + 2^10 + 1)
+    return np.full(shape, (300 * 2.0 ** 30 - 512 * (2.0 ** 20 + 2.0 ** 10 + 1)) / 2.0 ** 38)
+
+
+@pytest.mark.parametrize("kind", ["normal", "largest", "aligned", "lowest"])
+@pytest.mark.parametrize("M,N,K", SIZES)
+def test_digits_and_tiles(sc, M, N, K, kind):
+    rng = np.random.default_rng(M + 7 * N + 13 * K)
+    p = sc.Plan("ij,jk->ik", (1,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
+    assert p.info.tensor_core == 1
+    u, v = draw(kind, (M, K), rng), np.ascontiguousarray(draw(kind, (N, K), rng).T)
+    w = p.contract(torch.from_numpy(u).cuda().reshape(p.shape_u), torch.from_numpy(v).cuda().reshape(p.shape_v))
+    torch.cuda.synchronize()
+    p.check_device_error()
+    got = w.cpu().numpy().reshape(M, N)
+    scale = lambda x, axis: 2.0 ** np.ceil(np.log2(np.abs(x).max(axis) * (1 + 2.0 ** -50)))
+    bound = K * 2.0 ** -36 * np.outer(scale(u, 1), scale(v, 0))
+    assert np.all(np.abs(got - u @ v) <= bound + 1e-15 * (np.abs(u) @ np.abs(v)))
+
+
+def test_exact_products_at_the_sum_limits(sc):
+    """Entries +-1 and small multiples of 2^-9: two digits each, so every product is
+    in the exact diagonals 0 to 2 and the result is the exact sum."""
+    rng = np.random.default_rng(3)
+    M, N, K = 130, 70, 20000
+    u, v = (rng.choice([1.0, -1.0, 2.0 ** -9, 3.0 * 2.0 ** -9], (r, K)) for r in (M, N))
+    u[:, 0] = v[:, 0] = 1.0
+    p = sc.Plan("ij,jk->ik", (1,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
+    w = p.contract(torch.from_numpy(u).cuda().reshape(p.shape_u),
+                   torch.from_numpy(np.ascontiguousarray(v.T)).cuda().reshape(p.shape_v))
+    ui, vi = (np.rint(x * 2.0 ** 9).astype(np.int64) for x in (u, v))
+    exact = (ui @ vi.T).astype(np.float64) * 2.0 ** -18    # |sum| < 2^53
+    assert np.array_equal(w.cpu().numpy().reshape(M, N), exact)
