@@ -247,6 +247,9 @@ struct symctr_plan {
   int s = 0, t = 0, vv = 0, sigma = -1;
   std::vector<int> FU, C, FV;  // mode positions: FU, C in U; FV in V
   Problem prob;
+  // the problem the kernels run: `prob`, in a general plan without the aligned
+  // rows and columns that no irrep has (compact_tables)
+  Problem run;
   int64_t numel_u = 0, numel_v = 0, numel_w = 0;
   symctr_precision prec = SYMCTR_FP64;
   int n_slices = 0;
@@ -281,9 +284,11 @@ struct symctr_plan {
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   mutable int last_launches = 0;
   // offset tables of all irreps (tensor-core forms and general plans),
-  // computed once on the host in the workspace layout of a single pass;
-  // page-locked on first use
+  // computed once on the host in the workspace layout of a single pass of `run`;
+  // page-locked on first use.  From whole_tab on (general plans that dropped
+  // rows or columns; else 0) follow the tables of `prob`, for symctr_align.
   std::vector<int64_t> htab;
+  int64_t whole_tab = 0;
   mutable std::once_flag pin_once;
   mutable bool pinned = false;
   mutable const int64_t* dtab = nullptr;   // device view of the page-locked tables
@@ -412,6 +417,76 @@ int64_t gcd64(int64_t a, int64_t b) {
     b = t;
   }
   return a;
+}
+
+// Sets P->run (and kpad) and P->htab from `whole`, the tables of P->prob.  Under
+// sub-group coefficients or padded sectors most aligned indices of an irrep may
+// be absent (offset -1): a contracted mode pair of 8 and 2 sectors has one
+// solvable pair in four, blocks half full leave a quarter of each pair.  The
+// rows, columns and contracted indices present on both of their tensors move to
+// the front, irrep by irrep, and M, N and K shrink to the largest count; -1
+// fills the other irreps up.  (Absent entries of W are zeros that the zero fill
+// writes.)  The ladder with 8 x 24 virtual, 8 x 8 occupied indices, sub-group
+// modes and ragged sectors: 4608 x 512 x 4608 -> 1285 x 192 x 738 per irrep, 2.32 -> 0.13 ms.
+void compact_tables(symctr_plan* P, std::vector<int64_t>& whole) {
+  const Problem& pr = P->prob;
+  P->run = pr;
+  P->whole_tab = 0;
+  P->kpad = round_up(pr.K, kKBlock);
+  // only where the zero fill covers all of W
+  if (!P->fill_all) {
+    P->htab.swap(whole);
+    return;
+  }
+  const int64_t ext[6] = {pr.M, pr.K, pr.N, pr.K, pr.M, pr.N};
+  const int64_t* t[6];
+  const int64_t* at = whole.data();
+  for (int k = 0; k < 6; ++k) {
+    t[k] = at;
+    at += (int64_t)pr.n_q * ext[k];
+  }
+  const int pair[3][2] = {{0, 4}, {2, 5}, {1, 3}};   // (U, W) rows, (V, W) columns, contracted
+  int64_t len[3] = {1, 1, 1};
+  for (int a = 0; a < 3; ++a)
+    for (int b = 0; b < pr.n_q; ++b) {
+      const int64_t n = ext[pair[a][0]];
+      int64_t have = 0;
+      for (int64_t r = 0; r < n; ++r) have += t[pair[a][0]][b * n + r] >= 0 && t[pair[a][1]][b * n + r] >= 0;
+      if (have > len[a]) len[a] = have;
+    }
+  if (len[0] == pr.M && len[1] == pr.N && len[2] == pr.K) {
+    P->htab.swap(whole);
+    return;
+  }
+  P->run.M = len[0];
+  P->run.N = len[1];
+  P->run.K = len[2];
+  P->kpad = round_up(P->run.K, kKBlock);
+  const int64_t clen[6] = {len[0], len[2], len[1], len[2], len[0], len[1]};
+  const int64_t n_run = tables_entries(P->run);
+  std::vector<int64_t> tab((size_t)n_run, -1);
+  int64_t* dst[6];
+  int64_t* d = tab.data();
+  for (int k = 0; k < 6; ++k) {
+    dst[k] = d;
+    d += (int64_t)pr.n_q * clen[k];
+  }
+  for (int a = 0; a < 3; ++a)
+    for (int b = 0; b < pr.n_q; ++b) {
+      const int x = pair[a][0], y = pair[a][1];
+      const int64_t n = ext[x];
+      int64_t j = (int64_t)b * len[a];
+      for (int64_t r = 0; r < n; ++r) {
+        const int64_t ox = t[x][b * n + r], oy = t[y][b * n + r];
+        if (ox < 0 || oy < 0) continue;
+        dst[x][j] = ox;
+        dst[y][j] = oy;
+        ++j;
+      }
+    }
+  P->whole_tab = n_run;
+  tab.insert(tab.end(), whole.begin(), whole.end());
+  P->htab.swap(tab);
 }
 
 symctr_status build(const char* einsum, int n_moduli, const int32_t* moduli, const OpDesc& du_,
@@ -684,17 +759,19 @@ symctr_status build(const char* einsum, int n_moduli, const int32_t* moduli, con
     return bail(SYMCTR_ERR_ARGUMENT, "split form needs at least 2 slices");
   P->kpad = round_up(pr.K, kKBlock);
   pr.q_base = 0;
+  P->run = pr;
   if (P->tensor_core || (P->general && pr.n_q > 0)) {
     // the six offset tables [U rows | U cols | V rows | V cols | W rows | W cols],
     // each [n_q][extent]: the same function of the plan on every call
     const int64_t total = tables_entries(pr);
     if (total > (int64_t)1 << 28) return bail(SYMCTR_ERR_OVERFLOW, "offset tables too large");
+    std::vector<int64_t> tab;
     try {
-      P->htab.resize((size_t)total);
+      tab.resize((size_t)total);
     } catch (const std::bad_alloc&) {
       return bail(SYMCTR_ERR_OVERFLOW, "offset tables: host allocation failed");
     }
-    int64_t* t = P->htab.data();
+    int64_t* t = tab.data();
     const AxisMap* maps[6] = {&pr.u.rows, &pr.u.cols, &pr.v.rows, &pr.v.cols, &pr.w.rows, &pr.w.cols};
     const int64_t ext[6] = {pr.M, pr.K, pr.N, pr.K, pr.M, pr.N};
     for (int k = 0; k < 6; ++k)
@@ -702,14 +779,19 @@ symctr_status build(const char* einsum, int n_moduli, const int32_t* moduli, con
         for (int64_t r = 0; r < ext[k]; ++r)
           *t++ = P->general ? gen_offset(gax[k], pr.g, batch_irrep(pr, b), r)
                             : axis_offset(*maps[k], pr.g, batch_irrep(pr, b), r);
+    try {
+      compact_tables(P, tab);
+    } catch (const std::bad_alloc&) {
+      return bail(SYMCTR_ERR_OVERFLOW, "offset tables: host allocation failed");
+    }
   }
   {
-    Layout full = make_layout(pr, P->tensor_core, P->general, prec, P->n_slices, P->kpad);
+    Layout full = make_layout(P->run, P->tensor_core, P->general, prec, P->n_slices, P->kpad);
     if (!full.ok) return bail(SYMCTR_ERR_OVERFLOW, "aligned operand too large");
     P->ws_bytes = full.bytes;
     P->ws_bytes_min = full.bytes;
     if (P->tensor_core && pr.q_single < 0 && pr.n_q > 1) {
-      Problem one = pr;
+      Problem one = P->run;
       one.n_q = 1;
       P->ws_bytes_min = make_layout(one, true, P->general, prec, P->n_slices, P->kpad).bytes;
     }
@@ -900,7 +982,7 @@ bool tables_attached(const symctr_plan* P) {
 // tiles, are copied to HBM instead), or a copy into the workspace at off_tab.
 symctr_status pass_tables(const symctr_plan* P, const Problem& pc, int q0, bool attached, char* base,
                           uint64_t off_tab, cudaStream_t st, Tables* tab) {
-  const Problem& pr = P->prob;
+  const Problem& pr = P->run;
   const int64_t ext[6] = {pr.M, pr.K, pr.N, pr.K, pr.M, pr.N};
   const int64_t* in_place = attached ? P->dev_tab
                             : (P->dtab && P->htab.size() * sizeof(int64_t) <= kMappedTablesMax)
@@ -925,7 +1007,8 @@ symctr_status pass_tables(const symctr_plan* P, const Problem& pc, int q0, bool 
   tab->wcol = tab->wrow + (int64_t)pc.n_q * pc.M;
   cudaError_t e = cudaSuccess;
   if (pc.n_q == pr.n_q) {
-    e = cudaMemcpyAsync(t0, P->htab.data(), P->htab.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st);
+    e = cudaMemcpyAsync(t0, P->htab.data(), (size_t)tables_entries(pr) * sizeof(int64_t),
+                        cudaMemcpyHostToDevice, st);
   } else {
     const int64_t* src = P->htab.data();
     int64_t* dst = t0;
@@ -942,7 +1025,7 @@ symctr_status pass_tables(const symctr_plan* P, const Problem& pc, int q0, bool 
 symctr_status run_contract_body(const symctr_plan* P, const double* u, const double* v,
                                 double* w, void* ws, size_t ws_bytes, cudaStream_t st,
                                 const RunMode& mode) {
-  Problem prob = P->prob;
+  Problem prob = P->run;
   prob.es = mode.es;
   prob.negate = mode.negate;
   prob.accumulate = mode.accumulate;
@@ -1359,6 +1442,7 @@ symctr_status symctr_align(const symctr_plan* P, int operand, int direction, con
   if (!attached) pin_tables(P);
   const int64_t* t0 = attached ? P->dev_tab : P->dtab;
   if (!t0) return fail(SYMCTR_ERR_CUDA, "offset tables could not be mapped; attach them first");
+  t0 += P->whole_tab;
   tab.urow = t0;
   tab.ucol = tab.urow + (int64_t)pr.n_q * pr.M;
   tab.vrow = tab.ucol + (int64_t)pr.n_q * pr.K;
@@ -1538,6 +1622,7 @@ symctr_status symctr_plan_chain(symctr_plan* P, const symctr_plan* u_from, const
   Problem& pr = P->prob;
   GenAxis gax[6];
   plan_axes(P, gax);
+  std::vector<int64_t> whole;
   if (pr.n_q > 0) {
     const int64_t total = tables_entries(pr);
     if (total > (int64_t)1 << 28) return fail(SYMCTR_ERR_OVERFLOW, "offset tables too large");
@@ -1565,20 +1650,26 @@ symctr_status symctr_plan_chain(symctr_plan* P, const symctr_plan* u_from, const
           *t++ = off;
         }
       }
-    P->htab.swap(tab);
+    whole.swap(tab);
   }
   P->chained = true;
   P->general = true;
   pr.general = 1;
+  try {
+    if (pr.n_q > 0) compact_tables(P, whole);
+    else P->run = pr;
+  } catch (const std::bad_alloc&) {
+    return fail(SYMCTR_ERR_OVERFLOW, "offset tables: host allocation failed");
+  }
   P->row_run[0] = P->row_run[1] = 0;
   if (u_from) P->numel_u = (int64_t)u_from->prob.n_q * u_from->prob.M * u_from->prob.N;
   if (v_from) P->numel_v = (int64_t)v_from->prob.n_q * v_from->prob.M * v_from->prob.N;
   if (w_aligned) P->numel_w = (int64_t)pr.n_q * pr.M * pr.N;
-  Layout full = make_layout(pr, P->tensor_core, true, P->prec, P->n_slices, P->kpad);
+  Layout full = make_layout(P->run, P->tensor_core, true, P->prec, P->n_slices, P->kpad);
   if (!full.ok) return fail(SYMCTR_ERR_OVERFLOW, "aligned operand too large");
   P->ws_bytes = P->ws_bytes_min = full.bytes;
   if (P->tensor_core && pr.q_single < 0 && pr.n_q > 1) {
-    Problem one = pr;
+    Problem one = P->run;
     one.n_q = 1;
     P->ws_bytes_min = make_layout(one, true, true, P->prec, P->n_slices, P->kpad).bytes;
   }

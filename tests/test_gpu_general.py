@@ -154,3 +154,28 @@ def test_general_backward(sc, precision):
     plan.check_device_error()
     assert rel(gu.cpu().numpy(), O.grad_u(p, gw, v)) <= TOL[precision]
     assert rel(gv.cpu().numpy(), O.grad_v(p, u, gw)) <= TOL[precision]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "split_bf16", "tf32"])
+def test_general_dropped_rows_on_every_route(sc, precision):
+    """General plans run without the aligned rows and columns that no irrep has:
+    the same results from tables read in host memory or copied into the workspace
+    (static scratch), attached, and irrep by irrep in the smallest workspace; a
+    sector count that differs by irrep leaves absent rows in some of them."""
+    rng = np.random.default_rng(6500)
+    for G, dv, do in [(8, 12, 6), (6, 5, 3), (4, 9, 4)]:
+        p, u, v = cc_like(rng, G=G, dv=dv, do=do)
+        plan = sc.Plan(f"{p.lu},{p.lv}->{p.lw}", p.group.moduli, as_spec(p.sym_u), as_spec(p.sym_v), precision)
+        i = plan.info
+        whole = 8 * i.n_q * (2 * i.M + 2 * i.N + 2 * i.K) + (0 if precision == "fp64" else 4 * i.n_q * (i.M + i.N) * i.K)
+        assert i.workspace_bytes < whole // 2
+        want = O.contract_blockloop(p, u, v)
+        ud, vd = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+        first = plan.contract_static_scratch(ud, vd)     # no tables attached yet
+        plan.check_static_scratch_error()
+        assert rel(first.cpu().numpy(), want) <= TOL[precision]
+        ws = torch.empty(int(i.workspace_bytes_min), dtype=torch.uint8, device="cuda")
+        for w in (plan.contract(ud, vd), plan.contract(ud, vd, workspace=ws)):
+            assert rel(w.cpu().numpy(), want) <= TOL[precision]
+        plan.check_device_error()
+        plan.check_device_error(ws)
