@@ -21,7 +21,7 @@ namespace symctr {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, THREADS = 256;
+constexpr int BK = 16, THREADS = 256;
 
 // axis_offset as one out-of-line device function: every kernel below computes
 // offsets in a dozen places (per instance of the short-side row count), and
@@ -36,97 +36,137 @@ __host__ __device__ inline bool map_rows_fast(const AxisMap& rows) {
   return rows.n > 0 && rows.bstride[rows.n - 1] == 1;
 }
 
+// GEMM-shaped problems, T x T output tiles by 256 threads: (T / 16)^2 outputs a
+// thread, or (T = 8) one output by four threads that split each K block.  The
+// float64 pipe (2 FMAs per SM and clock) is the bound at every T: what matters
+// is that all SMs have the same share, and that a small problem has tiles for
+// all of them (tile_choice): 48 x 48 x 48 by 3 irreps ran on three SMs with
+// 64 x 64 tiles, 65 -> 17 us (launch-bound) with 8 x 8; the two MPS contractions
+// 128 x 2048 x 128 and 128 x 128 x 2048 by 8 irreps, on 3.4 tiles per SM and on
+// 128 of 152 SMs, 1177 -> 951 us with 32 x 32 and 7 K ranges (909 us at the
+// float64 rate of a large product).  Column offsets are computed for kKc columns of K
+// at a time, one per thread; the next K block's gathers are in flight while
+// this one is multiplied.
 // General plans pass their offset tables (t.urow != NULL): offsets come from
 // them, -1 marking an absent aligned row or column (read as zero, not stored).
-__global__ void __launch_bounds__(THREADS) gemm_f64_tiled(const __grid_constant__ Problem p, int ksplit, bool u_rows_fast,
-                                                          bool v_rows_fast, const Tables t,
-                                                          const double* __restrict__ U,
-                                                          const double* __restrict__ V,
-                                                          double* __restrict__ W) {
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
-  __shared__ int64_t uoff[BM], voff[BN], kuoff[BK], kvoff[BK], woffr[BM], woffc[BN];
+constexpr int kKc = 256;
+
+template <int T>
+__global__ void __launch_bounds__(THREADS) gemm_f64_tiled(const __grid_constant__ Problem p, int ksplit,
+                                                          int64_t kchunk, bool u_rows_fast, bool v_rows_fast,
+                                                          const Tables t, const double* __restrict__ U,
+                                                          const double* __restrict__ V, double* __restrict__ W) {
+  constexpr int R = T >= 16 ? T / 16 : 1;                      // outputs per thread and side
+  constexpr int NL = (T * BK + THREADS - 1) / THREADS;         // gathers per thread, operand and K block
+  __shared__ double As[2][BK][T + 1];
+  __shared__ double Bs[2][BK][T + 1];
+  __shared__ int64_t uoff[T], voff[T], woffr[T], woffc[T], ku[kKc], kv[kKc];
   const int tid = threadIdx.x;
-  const int tr = tid / 16, tc = tid % 16;
-  const int64_t mt = (p.M + BM - 1) / BM, nt = (p.N + BN - 1) / BN;
-  const int64_t kchunk = ((p.K + ksplit - 1) / ksplit + BK - 1) / BK * BK;
+  const int tr = T >= 16 ? tid / 16 : (tid & 63) / 8, tc = T >= 16 ? tid % 16 : tid % 8;
+  const int64_t mt = (p.M + T - 1) / T, nt = (p.N + T - 1) / T;
   const int64_t ntiles = mt * nt * p.n_q * ksplit;
+  const bool tab = t.urow != nullptr;
   for (int64_t tI = blockIdx.x; tI < ntiles; tI += gridDim.x) {
-    int64_t ks = tI % ksplit;
-    int64_t t2 = tI / ksplit;
-    int64_t b = t2 / (mt * nt);
-    int64_t rem = t2 - b * mt * nt;
-    int64_t m0 = (rem / nt) * BM, n0 = (rem % nt) * BN;
-    int Q = batch_irrep(p, (int)b);
-    int64_t kbeg = ks * kchunk, kend = kbeg + kchunk < p.K ? kbeg + kchunk : p.K;
+    const int64_t ks = tI % ksplit;
+    const int64_t t2 = tI / ksplit;
+    const int64_t b = t2 / (mt * nt);
+    const int64_t rem = t2 - b * mt * nt;
+    const int64_t m0 = (rem / nt) * T, n0 = (rem % nt) * T;
+    const int Q = batch_irrep(p, (int)b);
+    const int64_t kbeg = ks * kchunk, kend = kbeg + kchunk < p.K ? kbeg + kchunk : p.K;
     __syncthreads();
-    const bool tab = t.urow != nullptr;
-    if (tid < BM) {
-      int64_t m = m0 + tid;
-      uoff[tid] = m >= p.M ? 0 : tab ? t.urow[b * p.M + m] : aoff(p.u.rows, p.g, Q, m);
-      woffr[tid] = m >= p.M ? 0 : tab ? t.wrow[b * p.M + m] : aoff(p.w.rows, p.g, Q, m);
-    } else if (tid < BM + BN) {
-      int64_t n = n0 + tid - BM;
-      voff[tid - BM] = n >= p.N ? 0 : tab ? t.vrow[b * p.N + n] : aoff(p.v.rows, p.g, Q, n);
-      woffc[tid - BM] = n >= p.N ? 0 : tab ? t.wcol[b * p.N + n] : aoff(p.w.cols, p.g, Q, n);
+    if (tid < T) {
+      const int64_t m = m0 + tid;
+      uoff[tid] = m >= p.M ? -1 : tab ? t.urow[b * p.M + m] : aoff(p.u.rows, p.g, Q, m);
+      woffr[tid] = m >= p.M ? -1 : tab ? t.wrow[b * p.M + m] : aoff(p.w.rows, p.g, Q, m);
+    } else if (tid >= 128 && tid < 128 + T) {
+      const int64_t n = n0 + tid - 128;
+      voff[tid - 128] = n >= p.N ? -1 : tab ? t.vrow[b * p.N + n] : aoff(p.v.rows, p.g, Q, n);
+      woffc[tid - 128] = n >= p.N ? -1 : tab ? t.wcol[b * p.N + n] : aoff(p.w.cols, p.g, Q, n);
     }
-    double acc[4][4];
+    double acc[R][R];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
+      for (int j = 0; j < R; ++j) acc[i][j] = 0.0;
+    for (int64_t kc = kbeg; kc < kend; kc += kKc) {
+      const int n = kend - kc < kKc ? (int)(kend - kc) : kKc;
       __syncthreads();
-      if (tid < BK) {
-        int64_t k = k0 + tid;
-        kuoff[tid] = k >= kend ? 0 : tab ? t.ucol[b * p.K + k] : aoff(p.u.cols, p.g, Q, k);
-      } else if (tid >= 32 && tid < 32 + BK) {
-        int64_t k = k0 + tid - 32;
-        kvoff[tid - 32] = k >= kend ? 0 : tab ? t.vcol[b * p.K + k] : aoff(p.v.cols, p.g, Q, k);
+      if (tid < n) {
+        const int64_t k = kc + tid;
+        ku[tid] = tab ? t.ucol[b * p.K + k] : aoff(p.u.cols, p.g, Q, k);
+        kv[tid] = tab ? t.vcol[b * p.K + k] : aoff(p.v.cols, p.g, Q, k);
       }
       __syncthreads();
+      double xa[NL], xb[NL];
+      auto gather = [&](int k0) {
 #pragma unroll
-      for (int j = 0; j < (BM * BK) / THREADS; ++j) {
-        int e = tid + j * THREADS;
-        int mm = u_rows_fast ? e % BM : e / BK;
-        int kk = u_rows_fast ? e / BM : e % BK;
-        double x = 0.0;
-        if (m0 + mm < p.M && k0 + kk < kend && uoff[mm] >= 0 && kuoff[kk] >= 0)
-          x = U[p.es * (uoff[mm] + kuoff[kk])];
-        As[kk][mm] = x;
-      }
+        for (int j = 0; j < NL; ++j) {
+          const int e = tid + j * THREADS;
+          xa[j] = xb[j] = 0.0;
+          if (e < T * BK) {
+            int mm = u_rows_fast ? e % T : e / BK, kk = k0 + (u_rows_fast ? e / T : e % BK);
+            if (kk < n && uoff[mm] >= 0 && ku[kk] >= 0) xa[j] = U[p.es * (uoff[mm] + ku[kk])];
+            mm = v_rows_fast ? e % T : e / BK, kk = k0 + (v_rows_fast ? e / T : e % BK);
+            if (kk < n && voff[mm] >= 0 && kv[kk] >= 0) xb[j] = V[p.es * (voff[mm] + kv[kk])];
+          }
+        }
+      };
+      auto stage = [&](int buf) {
 #pragma unroll
-      for (int j = 0; j < (BN * BK) / THREADS; ++j) {
-        int e = tid + j * THREADS;
-        int nn = v_rows_fast ? e % BN : e / BK;
-        int kk = v_rows_fast ? e / BN : e % BK;
-        double x = 0.0;
-        if (n0 + nn < p.N && k0 + kk < kend && voff[nn] >= 0 && kvoff[kk] >= 0)
-          x = V[p.es * (voff[nn] + kvoff[kk])];
-        Bs[kk][nn] = x;
-      }
+        for (int j = 0; j < NL; ++j) {
+          const int e = tid + j * THREADS;
+          if (e < T * BK) {
+            As[buf][u_rows_fast ? e / T : e % BK][u_rows_fast ? e % T : e / BK] = xa[j];
+            Bs[buf][v_rows_fast ? e / T : e % BK][v_rows_fast ? e % T : e / BK] = xb[j];
+          }
+        }
+      };
+      gather(0);
+      stage(0);
       __syncthreads();
+      for (int k0 = 0, buf = 0; k0 < n; k0 += BK, buf ^= 1) {
+        if (k0 + BK < n) gather(k0 + BK);
+        if constexpr (T >= 16) {
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        double a[4], bb[4];
+          for (int kk = 0; kk < BK; ++kk) {
+            double a[R], bb[R];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][tr + 16 * i];
+            for (int i = 0; i < R; ++i) a[i] = As[buf][kk][tr + 16 * i];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tc + 16 * j];
+            for (int j = 0; j < R; ++j) bb[j] = Bs[buf][kk][tc + 16 * j];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+              for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < BK / 4; ++q) {
+            const int kk = (tid >> 6) * (BK / 4) + q;
+            acc[0][0] = fma(As[buf][kk][tr], Bs[buf][kk][tc], acc[0][0]);
+          }
+        }
+        if (k0 + BK < n) stage(buf ^ 1);
+        __syncthreads();
       }
     }
+    if constexpr (T < 16) {
+      double* red = &As[0][0][0];
+      static_assert(T >= 16 || sizeof(As) >= THREADS * sizeof(double), "reduction buffer");
+      red[tid] = acc[0][0];
+      __syncthreads();
+      if (tid < 64) acc[0][0] = (red[tid] + red[tid + 64]) + (red[tid + 128] + red[tid + 192]);
+      if (tid >= 64) continue;
+    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int mm = tr + 16 * i;
-      if (m0 + mm >= p.M || woffr[mm] < 0) continue;
+    for (int i = 0; i < R; ++i) {
+      const int mm = tr + 16 * i;
+      if (woffr[mm] < 0) continue;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        int nn = tc + 16 * j;
-        if (n0 + nn >= p.N || woffc[nn] < 0) continue;
+      for (int j = 0; j < R; ++j) {
+        const int nn = tc + 16 * j;
+        if (woffc[nn] < 0) continue;
         double* dst = W + p.es * (woffr[mm] + woffc[nn]);
         if (ksplit > 1) atomicAdd(dst, signed_result(p, acc[i][j]));
         else store_w(p, dst, acc[i][j]);
@@ -657,13 +697,44 @@ void launch_skinny_ns(int sms, cudaStream_t st, const Problem& p, bool long_is_u
   gemm_f64_skinny<NS><<<grid, THREADS, 0, st>>>(p, long_is_u, (int)ksplit, u, v, w);
 }
 
+// Tile and K ranges of the tiled kernel: the least time of the busiest SM.  A K
+// block of a T x T tile takes 8 T^2 clocks of the float64 pipe, and about 1000
+// clocks more (offsets, gathers, barriers) when an SM has one tile at a time,
+// 200 when several share it.  K ranges (at least 256 columns) cost a zeroed W
+// and atomic adds: about 6000 clocks.
+struct TileChoice {
+  int T = 64, ksplit = 1;
+  int64_t kchunk = 0, units = 0;
+};
+TileChoice tile_choice(const Problem& p, int sms) {
+  TileChoice best;
+  double least = 0;
+  for (int T : {64, 32, 16, 8}) {
+    const int64_t tiles = ((p.M + T - 1) / T) * ((p.N + T - 1) / T) * p.n_q;
+    for (int s = 1; s <= 16 && (s == 1 || p.K / s >= 256); ++s) {
+      const int64_t blocks = ((p.K + s - 1) / s + BK - 1) / BK;   // K blocks of a range
+      const int64_t ranges = (p.K + blocks * BK - 1) / (blocks * BK);
+      const int64_t units = tiles * ranges, rounds = (units + sms - 1) / sms;
+      const double time = (double)rounds * blocks * (8.0 * T * T + (units > sms ? 200 : 1000)) +
+                          (ranges > 1 ? 6000 : 0);
+      if (best.units == 0 || time < 0.97 * least) {
+        least = time;
+        best.T = T;
+        best.ksplit = (int)ranges;
+        best.kchunk = blocks * BK;
+        best.units = units;
+      }
+    }
+  }
+  return best;
+}
+
 }  // namespace
 
 cudaError_t launch_gemm_f64(const Problem& p, const double* u, const double* v, double* w,
                             const Tables* tables, cudaStream_t st) {
   if (p.n_q == 0 || p.M == 0 || p.N == 0) return cudaSuccess;
   const int sms = sm_count();
-  const int64_t target = (int64_t)sms * 2;
   // general plans take the tiled kernel with their tables (every shape)
   bool skinny = !tables && (p.M < 16 || p.N < 16);
   if (skinny && (p.M <= SKINNY_MAX || p.N <= SKINNY_MAX)) {
@@ -703,20 +774,19 @@ cudaError_t launch_gemm_f64(const Problem& p, const double* u, const double* v, 
     ++g_kernel_launches;
     return cudaGetLastError();
   }
-  int64_t tiles = ((p.M + BM - 1) / BM) * ((p.N + BN - 1) / BN) * p.n_q;
-  int ksplit = 1;
-  while (tiles * ksplit < target && p.K / (ksplit * 2) >= 512) ksplit *= 2;
+  const TileChoice c = tile_choice(p, sms);
   // (a general plan's W is zeroed as a whole before its contraction)
-  if (ksplit > 1 && !p.accumulate && !tables) {
+  if (c.ksplit > 1 && !p.accumulate && !tables) {
     zero_w_entries<<<sms * 4, 256, 0, st>>>(p, w);
     ++g_kernel_launches;
   }
   Tables t{};
   if (tables) t = *tables;
-  int64_t blocks = tiles * ksplit;
-  int64_t cap = (int64_t)sms * 4;
-  gemm_f64_tiled<<<(int)(blocks < cap ? blocks : cap), THREADS, 0, st>>>(
-      p, ksplit, map_rows_fast(p.u.rows), map_rows_fast(p.v.rows), t, u, v, w);
+  auto kern = c.T == 64 ? gemm_f64_tiled<64> : c.T == 32 ? gemm_f64_tiled<32> : c.T == 16 ? gemm_f64_tiled<16>
+                                                                                      : gemm_f64_tiled<8>;
+  const int64_t cap = (int64_t)sms * 4;
+  kern<<<(int)(c.units < cap ? c.units : cap), THREADS, 0, st>>>(
+      p, c.ksplit, c.kchunk, map_rows_fast(p.u.rows), map_rows_fast(p.v.rows), t, u, v, w);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
