@@ -29,7 +29,8 @@
 // side: one MMA per A digit takes all the B digits it pairs with (N = 256, 192,
 // 128, 64).  Each half has its own issuing thread and its own 8 warps, so that
 // its drain (TMEM loads, FP32 and integer adds) runs beside the other half's
-// MMAs.  A half beyond N is neither loaded nor multiplied.
+// MMAs.  A half beyond N is neither loaded nor multiplied.  Where the wide tiles
+// would leave SMs idle, a 128 x 64 tile is a CTA of its own, two to an SM.
 //
 // What bounds it: a stage's operands cross shared memory at 128 B/clk, 64 KB
 // written by TMA and 144 KB read by the MMAs (1664 clocks; the MMAs alone would
@@ -48,24 +49,29 @@ namespace symctr {
 namespace {
 
 constexpr int TM = 128;
-constexpr int TN = 128;
 constexpr int HN = 64;            // columns of a half tile
-constexpr int NTHREADS = 640;
-constexpr int EPI_WARPS = 16;
 constexpr int EPI_WARP0 = 4;
 constexpr int P4 = 4;             // digit planes
 constexpr int ROWB = 64;          // bytes per tile row and stage: 32 FP16, SWIZZLE_64B
 constexpr int KSTAGE = 32;
-constexpr int STAGES = 3;
 constexpr int kFold = 16;         // stages between folds of diagonal 2 (even)
 constexpr int A_BYTES = P4 * TM * ROWB;     // all digits of a stage's A tile
-constexpr int B_BYTES = P4 * HN * ROWB;     // of half a B tile
-constexpr int STAGE_BYTES = A_BYTES + 2 * B_BYTES;
-constexpr int LD = TN + 1;        // epilogue staging stride (doubles)
-constexpr size_t REGION = (size_t)STAGES * STAGE_BYTES;
-static_assert(REGION >= (size_t)TM * LD * 8, "the epilogue staging fits the stages");
-constexpr int BARS = 2 * STAGES + 6;
-constexpr size_t SMEM = 1024 + REGION + 8 * BARS + 12 * (TN + TM) + 16 + 64;
+constexpr int B_BYTES = P4 * HN * ROWB;     // of one half's B tile
+
+// H = 2: both halves, one CTA per SM; H = 1: a 128 x 64 tile, two CTAs per SM.
+template <int H>
+struct Cfg {
+  static constexpr int TN = H * HN;
+  static constexpr int EPI_WARPS = 8 * H;
+  static constexpr int NTHREADS = 128 + 32 * EPI_WARPS;
+  static constexpr int STAGES = H == 2 ? 3 : 2;
+  static constexpr int STAGE_BYTES = A_BYTES + H * B_BYTES;
+  static constexpr int LD = TN + 1;        // epilogue staging stride (doubles)
+  static constexpr size_t REGION = (size_t)STAGES * STAGE_BYTES;
+  static_assert(REGION >= (size_t)TM * LD * 8, "the epilogue staging fits the stages");
+  static constexpr int BARS = 2 * STAGES + 6;
+  static constexpr size_t SMEM = 1024 + REGION + 8 * BARS + 12 * (TN + TM) + 16 + 64;
+};
 
 // K-major rows of 64 bytes, SWIZZLE_64B, 8-row groups 512 bytes apart.
 __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
@@ -118,17 +124,18 @@ struct Tc10Args {
   const int64_t* wcol;       // [n_q][N] offsets of W's columns
 };
 
-__device__ __forceinline__ int32_t f2i(uint32_t bits) { return __float2int_rn(__uint_as_float(bits)); }
-
-template <bool GEN>
-__global__ void __launch_bounds__(NTHREADS, 1)
+template <int H, bool GEN>
+__global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
     gemm_tc10_kernel(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b,
                      const __grid_constant__ Tc10Args args) {
+  using C = Cfg<H>;
+  constexpr int TN = C::TN, STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, LD = C::LD;
+  constexpr int EPI_WARPS = C::EPI_WARPS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const Problem& p = args.p;
   uint8_t* tiles = smem;  // [STAGES][A digits, B digits of half 0, of half 1], later the epilogue staging
-  uint64_t* full = (uint64_t*)(smem + REGION);
+  uint64_t* full = (uint64_t*)(smem + C::REGION);
   uint64_t* empty = full + STAGES;
   uint64_t* go = empty + STAGES;         // [2] a half's MMAs of a stage are done: drain
   uint64_t* drained = go + 2;            // [2] its accumulators may be written again
@@ -147,7 +154,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const int ks = blockIdx.z % args.ksplit;
   const int kb0 = ks * args.kb_per_split;
   const int n_kb = min(args.n_kb, kb0 + args.kb_per_split) - kb0;
-  const int halves = p.N - n0 > HN ? 2 : 1;
+  const int halves = H == 2 && p.N - n0 > HN ? 2 : 1;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -165,7 +172,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(su32(tmem_slot))
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
+                 "n"(4 * TN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -173,14 +181,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const int et = (int)threadIdx.x - EPI_WARP0 * 32;   // epilogue thread
   if (et >= 0 && et < TM) {
     roffs[et] = m0 + et < p.M ? args.wrow[(int64_t)b * p.M + m0 + et] : -1;
-    coff[et] = n0 + et < p.N ? args.wcol[(int64_t)b * p.N + n0 + et] : -1;
+    if (et < TN) coff[et] = n0 + et < p.N ? args.wcol[(int64_t)b * p.N + n0 + et] : -1;
   }
   // Launched as a programmatic dependent of the operand preparation: the setup
   // above overlaps its tail; everything below reads its outputs.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (et >= 0 && et < TM) {
     rexps[et] = m0 + et < p.M ? args.eu[(int64_t)b * p.M + m0 + et] - kExpBias : 0;
-    cexp[et] = n0 + et < p.N ? args.ev[(int64_t)b * p.N + n0 + et] - kExpBias : 0;
+    if (et < TN) cexp[et] = n0 + et < p.N ? args.ev[(int64_t)b * p.N + n0 + et] - kExpBias : 0;
   }
   tc_fence_before();
   __syncthreads();
@@ -188,8 +196,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const uint32_t tmem = *tmem_slot;
 
   // registers: part of the producer warpgroup's share goes to the running sums
-  // (56 x 128 + 104 x 512, less than the 96 x 640 that the CTA was launched with)
-  if (warp < EPI_WARP0) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+  // (H = 2: 56 x 128 + 104 x 512, less than the 96 x 640 of the launch; H = 1:
+  // 32 x 128 + 104 x 256, the 80 x 384 of the launch)
+  if (warp < EPI_WARP0) {
+    if constexpr (H == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    else asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+  }
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
@@ -268,6 +280,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int j = 0; j < 32; ++j) s0[j] = s1[j] = 0;
     const float M8 = 100663296.0f;             // 1.5 * 2^26: ulp 8, |x| <= 2^25
     const int32_t B8 = (int32_t)__float_as_uint(M8);
+    const float M0 = 12582912.0f;              // 1.5 * 2^23: ulp 1
+    const int32_t B0 = (int32_t)__float_as_uint(M0);
     // s += a's multiples of 8, a = what is left
     auto drain16 = [&](uint32_t* a, int32_t* s) {
 #pragma unroll
@@ -299,7 +313,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (o != 0 && (kb + 1) % kFold == 0) {
         // diagonal 2 (the MMAs that write it wait): multiples of 2^13 = 8 x 2^10
         // to s1, |rest| <= 2^12 stays
-        const float M0 = 12582912.0f;   // 1.5 * 2^23: ulp 1
 #pragma unroll
         for (int pc = 0; pc < 2; ++pc) {
           tmem_ld16(lane_base + 2 * HN + pc * 16, a);
@@ -310,7 +323,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const float x = __uint_as_float(a[j]);
             const float r = __fmaf_rn(x, 1.0f / 8192.0f, M0);   // round(x / 2^13) + 1.5 * 2^23
             int32_t& t = s1[pc * 16 + j];
-            t += (int32_t)__float_as_uint(r) - (int32_t)__float_as_uint(M0);
+            t += (int32_t)__float_as_uint(r) - B0;
             a[j] = __float_as_uint(__fmaf_rn(r - M0, -8192.0f, x));   // exact
             s0[pc * 16 + j] += t >> 10;
             t &= 1023;
@@ -364,13 +377,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tmem_loaded<4>(a3);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int32_t q0 = f2i(a0[j]), q1 = f2i(a1[j]);
-          const int32_t t3 = __float2int_rn(__uint_as_float(a3[j]) * (1.0f / 1024.0f));
-          // 32-bit sums with the last stage first: the 64-bit words of all
-          // columns at once would not fit the registers
-          const int32_t rest = ((q0 & 7) << 20) + ((q1 & 7) << 10) + f2i(a2[j]) + t3;
-          st64[pc * 4 + j] = ((long long)(s0[pc * 4 + j] + (q0 >> 3)) << 23) +
-                             ((long long)(s1[pc * 4 + j] + (q1 >> 3)) << 13) + rest;
+          // multiples of 8 of the exact diagonals by the magic number, as in the
+          // drains, their rests (an integer below 2^13) likewise; diagonals 2 and 3
+          // (|.| < 2^29) as one FP32 number and the only conversion
+          const float x0 = __uint_as_float(a0[j]), x1 = __uint_as_float(a1[j]);
+          const float r0 = x0 + M8, r1 = x1 + M8;
+          const int32_t t0 = s0[pc * 4 + j] + ((int32_t)__float_as_uint(r0) - B8);
+          const int32_t t1 = s1[pc * 4 + j] + ((int32_t)__float_as_uint(r1) - B8);
+          const float low = __fmaf_rn(__uint_as_float(a3[j]), 1.0f / 1024.0f, __uint_as_float(a2[j]));
+          const float rest = __fmaf_rn(x0 - (r0 - M8), 1024.0f, x1 - (r1 - M8));
+          const int32_t l = (((int32_t)__float_as_uint(rest + M0) - B0) << 10) + __float2int_rn(low);
+          st64[pc * 4 + j] = ((long long)t0 << 23) + ((long long)t1 << 13) + l;
         }
       }
     }
@@ -378,7 +395,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // all epilogue threads meet here, whatever path they took
     asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
     if (ok) {
-      // a warp per row: lane l rounds and writes columns l, l + 32, l + 64, l + 96
+      // a warp per row: lane l rounds and writes columns l, l + 32, ...; two rows
+      // at a time (one was bound by the latency of its conversions)
       constexpr int NC = TN / 32;
       const int nrow = (int)min((int64_t)TM, p.M - m0), ncol = (int)min((int64_t)TN, p.N - n0);
       const long long* R0 = (const long long*)tiles + lane;
@@ -396,7 +414,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         int ce[NC];
 #pragma unroll
         for (int j = 0; j < NC; ++j) co[j] = coff[lane + 32 * j], ce[j] = cexp[lane + 32 * j] - 36;
-#pragma unroll 1
+#pragma unroll 2
         for (int r = ew; r < nrow; r += EPI_WARPS) {
           const int64_t ro = roffs[r];
           const int re = rexps[r];
@@ -429,14 +447,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(4 * TN) : "memory");
   }
 }
 
-template <bool GEN>
+template <int H, bool GEN>
 cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, const void* bop, const int32_t* eu,
                         const int32_t* ev, int64_t kpad, double* w, unsigned* err, int ksplit,
                         unsigned long long* wacc, cudaStream_t st) {
+  using C = Cfg<H>;
+  constexpr int TN = C::TN;
   CUtensorMap ma, mb;
   if (!make_map(&ma, a, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, kpad, p.M, p.n_q, P4, KSTAGE, TM, P4) ||
       !make_map(&mb, bop, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, kpad, p.N, p.n_q, P4, KSTAGE, HN, P4))
@@ -454,12 +474,12 @@ cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, cons
   args.wacc = wacc;
   args.wrow = tab.wrow;
   args.wcol = tab.wcol;
-  auto kern = gemm_tc10_kernel<GEN>;
+  auto kern = gemm_tc10_kernel<H, GEN>;
   thread_local bool attr_set[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
   if (!attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
@@ -467,8 +487,8 @@ cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, cons
   if (gx > 0x7FFFFFFF || gy > 65535 || (int64_t)p.n_q * args.ksplit > 65535) return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)gx, (unsigned)gy, (unsigned)(p.n_q * args.ksplit));
-  cfg.blockDim = dim3(NTHREADS);
-  cfg.dynamicSmemBytes = SMEM;
+  cfg.blockDim = dim3(C::NTHREADS);
+  cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -481,14 +501,34 @@ cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, cons
   return launch_splitk_round(p, wacc, eu, ev, tab.wrow, tab.wcol, w, err, st);
 }
 
+template <int H>
+cudaError_t launch_tile(const Problem& p, const Tables& tab, const void* a, const void* bop, const int32_t* eu,
+                        const int32_t* ev, int64_t kpad, double* w, unsigned* err, int ksplit,
+                        unsigned long long* wacc, cudaStream_t st) {
+  if (p.es == 1 && !p.negate && !p.accumulate)
+    return launch_mode<H, false>(p, tab, a, bop, eu, ev, kpad, w, err, ksplit, wacc, st);
+  return launch_mode<H, true>(p, tab, a, bop, eu, ev, kpad, w, err, ksplit, wacc, st);
+}
+
 }  // namespace
 
 cudaError_t launch_gemm_split10(const Problem& p, const Tables& tab, const uint16_t* us, const uint16_t* vs,
                                 const int32_t* eu, const int32_t* ev, int64_t kpad, double* w, unsigned* err,
                                 int ksplit, unsigned long long* wacc, cudaStream_t st) {
-  if (p.es == 1 && !p.negate && !p.accumulate)
-    return launch_mode<false>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
-  return launch_mode<true>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
+  // The narrower tile where it takes fewer rounds of the SMs.  Clocks measured
+  // per stage and per tile: 1930 and 17000 for a 128 x 128 tile, 2270 and 20000
+  // for two 128 x 64 tiles side by side (they load the A digits twice: 4650
+  // against 4100 us for the CC ladder, but 1285 x 192 x 738 by 8 irreps, 176
+  // wide or 264 narrow tiles, takes 103 us instead of 129, preparation included).
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t split = ksplit < 1 ? 1 : ksplit, blocks = ((p.M + TM - 1) / TM) * p.n_q * split;
+  const int64_t n_kb = (kpad / KSTAGE + split - 1) / split;
+  const int64_t wide = blocks * ((p.N + 2 * HN - 1) / (2 * HN)), narrow = blocks * ((p.N + HN - 1) / HN);
+  const double t2 = (double)((wide + sms - 1) / sms) * (1930.0 * n_kb + 17000.0);
+  const double t1 = (double)((narrow + 2 * sms - 1) / (2 * sms)) * (2270.0 * n_kb + 20000.0);
+  if (t1 < 0.9 * t2) return launch_tile<1>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
+  return launch_tile<2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
 }
 
 }  // namespace symctr

@@ -68,3 +68,18 @@ def test_exact_products_at_the_sum_limits(sc):
     ui, vi = (np.rint(x * 2.0 ** 9).astype(np.int64) for x in (u, v))
     exact = (ui @ vi.T).astype(np.float64) * 2.0 ** -18    # |sum| < 2^53
     assert np.array_equal(w.cpu().numpy().reshape(M, N), exact)
+
+
+@pytest.mark.parametrize("M,N,K", [(2000, 190, 100), (1990, 129, 700), (2040, 192, 33)])
+def test_narrow_tiles(sc, M, N, K):
+    """Five irreps whose 128-column tiles need two rounds of the SMs and whose
+    64-column tiles need one: the narrow kernel."""
+    G = 5
+    p = sc.Plan("ij,jk->ik", (G,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
+    rng = np.random.default_rng(M)
+    u, v = rng.standard_normal(p.shape_u), rng.standard_normal(p.shape_v)
+    w = p.contract(torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()).cpu().numpy()
+    p.check_device_error()
+    for q in range(G):
+        bound = K * 2.0 ** -36 * 64.0    # |entries| < 8 = 2^(E+1)
+        assert np.all(np.abs(w[q] - u[q] @ v[q]) <= bound)
