@@ -295,7 +295,10 @@ SYMCTR_API symctr_status symctr_contract(const symctr_plan* plan, const double* 
  * conjugated operand is created with that operand's signs and charge negated
  * (its reduced array is the same).  Runs as four real contractions of the
  * plan's precision form on the real and imaginary parts (four times the real
- * work), with the same workspace and error reporting as symctr_contract.
+ * work), with the same workspace and error reporting as symctr_contract.  The
+ * default split form prepares each part once, in two GEMM launches, when the
+ * workspace holds both parts: 2 workspace_bytes + 16 n_q M N + 256 n_q (M + N) +
+ * 4096 bytes do.
  * Returns as symctr_contract. */
 SYMCTR_API symctr_status symctr_contract_complex(const symctr_plan* plan, int conj_u, int conj_v,
                                                 const double* u_red, const double* v_red,

@@ -363,6 +363,17 @@ class Plan:
             self._seen = set()   # the new buffer's streams are recorded afresh
         return self._ws
 
+    def _workspace_complex(self, device) -> torch.Tensor:
+        """The plan's workspace, grown to hold both parts of complex operands (each
+        part is then prepared once) where that takes at most 2 GiB."""
+        i = self.info
+        M, N, n_q = int(i.M), int(i.N), int(i.n_q)
+        need = 2 * int(i.workspace_bytes) + 16 * n_q * M * N + 256 * n_q * (M + N) + 4096
+        if need <= 2 << 30 and (self._ws is None or self._ws.numel() < need):
+            self._ws = torch.empty(need, dtype=torch.uint8, device=device or "cuda")
+            self._seen = set()
+        return self.workspace(device=device)
+
     # -- checks --------------------------------------------------------------
     @staticmethod
     def _dev64(t: torch.Tensor, shape, name):
@@ -416,7 +427,7 @@ class Plan:
         self._same_device(u, v, out, workspace)
         if not self._tables_ready:
             self.attach_tables(u.device)
-        ws = workspace if workspace is not None else self.workspace(device=u.device)
+        ws = workspace if workspace is not None else self._workspace_complex(u.device)
         self._used_on(torch.cuda.current_stream(), self._tables, self._ws)
         _check(load().symctr_contract_complex(self._h, int(conj_u), int(conj_v), _ptr(u), _ptr(v),
                                               _ptr(out), _ptr(ws), ws.numel(), _stream()))

@@ -867,7 +867,7 @@ cudaError_t launch_gemm_split(const Problem& p, const Tables& tab, int n_slices,
     case 2: return launch_tc<MODE_SPLIT, 2, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
     case 3: return launch_tc<MODE_SPLIT, 3, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
     case 4: return launch_tc<MODE_SPLIT, 4, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
-    case 5: return launch_gemm_split10(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
+    case 5: return launch_gemm_split10(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, nullptr, st);
     case 6: return launch_tc<MODE_SPLIT, 6, 2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
   }
   return cudaErrorInvalidValue;

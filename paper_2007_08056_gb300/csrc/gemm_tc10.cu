@@ -122,6 +122,11 @@ struct Tc10Args {
   unsigned long long* wacc;  // [n_q][M][N] int64 partial sums when ksplit > 1 (zeroed)
   const int64_t* wrow;       // [n_q][M] offsets of W's rows in its reduced form
   const int64_t* wcol;       // [n_q][N] offsets of W's columns
+  // Complex operands: the digits of real and imaginary parts are 2 n_q batches.
+  // One launch multiplies part upart of U by the `parts` parts of V (grid.z =
+  // parts * n_q * ksplit), part j into W + woff[j] with sign neg[j].
+  int parts, upart;
+  int woff[2], neg[2];
 };
 
 template <int H, bool GEN>
@@ -150,8 +155,10 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n0 = (int64_t)blockIdx.x * TN, m0 = (int64_t)blockIdx.y * TM;
-  const int b = blockIdx.z / args.ksplit;
+  const int zb = blockIdx.z / args.ksplit;       // part * n_q + irrep
   const int ks = blockIdx.z % args.ksplit;
+  const int part_v = zb >= p.n_q ? 1 : 0, b = zb - part_v * p.n_q;
+  const int ub = b + args.upart * p.n_q;         // U's batch (V's is zb)
   const int kb0 = ks * args.kb_per_split;
   const int n_kb = min(args.n_kb, kb0 + args.kb_per_split) - kb0;
   const int halves = H == 2 && p.N - n0 > HN ? 2 : 1;
@@ -187,8 +194,8 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
   // above overlaps its tail; everything below reads its outputs.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (et >= 0 && et < TM) {
-    rexps[et] = m0 + et < p.M ? args.eu[(int64_t)b * p.M + m0 + et] - kExpBias : 0;
-    if (et < TN) cexp[et] = n0 + et < p.N ? args.ev[(int64_t)b * p.N + n0 + et] - kExpBias : 0;
+    rexps[et] = m0 + et < p.M ? args.eu[(int64_t)ub * p.M + m0 + et] - kExpBias : 0;
+    if (et < TN) cexp[et] = n0 + et < p.N ? args.ev[(int64_t)zb * p.N + n0 + et] - kExpBias : 0;
   }
   tc_fence_before();
   __syncthreads();
@@ -213,9 +220,9 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
         uint8_t* sa = tiles + (size_t)st * STAGE_BYTES;
         // all four digit tiles of an operand in one copy
         const int kc = (kb0 + kb) * KSTAGE;
-        tma_load_4d(&tma_a, &full[st], sa, kc, (int)m0, b);
-        tma_load_4d(&tma_b, &full[st], sa + A_BYTES, kc, (int)n0, b);
-        if (halves == 2) tma_load_4d(&tma_b, &full[st], sa + A_BYTES + B_BYTES, kc, (int)n0 + HN, b);
+        tma_load_4d(&tma_a, &full[st], sa, kc, (int)m0, ub);
+        tma_load_4d(&tma_b, &full[st], sa + A_BYTES, kc, (int)n0, zb);
+        if (halves == 2) tma_load_4d(&tma_b, &full[st], sa + A_BYTES + B_BYTES, kc, (int)n0 + HN, zb);
         ++issued;
       }
       if (ctl->abort) {
@@ -401,7 +408,7 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
       const int nrow = (int)min((int64_t)TM, p.M - m0), ncol = (int)min((int64_t)TN, p.N - n0);
       const long long* R0 = (const long long*)tiles + lane;
       if (args.ksplit > 1) {
-        unsigned long long* acc = args.wacc + ((int64_t)b * p.M + m0) * p.N + n0 + lane;
+        unsigned long long* acc = args.wacc + ((int64_t)zb * p.M + m0) * p.N + n0 + lane;
 #pragma unroll 1
         for (int r = ew; r < nrow; r += EPI_WARPS) {
 #pragma unroll
@@ -410,6 +417,9 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
               red_add_u64(acc + (int64_t)r * p.N + 32 * j, (unsigned long long)R0[r * LD + 32 * j]);
         }
       } else {
+        OutMode wp;
+        wp.negate = args.neg[part_v];
+        wp.accumulate = p.accumulate;
         int64_t co[NC];
         int ce[NC];
 #pragma unroll
@@ -431,10 +441,7 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
             if constexpr (!GEN) {
               args.w[ro + co[j]] = d[j];
             } else {
-              double* at = args.w + (int64_t)p.es * (ro + co[j]);
-              const double x = signed_result(p, d[j]);
-              if (p.accumulate) *at += x;
-              else *at = x;
+              store_w(wp, args.w + args.woff[part_v] + (int64_t)p.es * (ro + co[j]), d[j]);
             }
           }
         }
@@ -454,12 +461,13 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
 template <int H, bool GEN>
 cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, const void* bop, const int32_t* eu,
                         const int32_t* ev, int64_t kpad, double* w, unsigned* err, int ksplit,
-                        unsigned long long* wacc, cudaStream_t st) {
+                        unsigned long long* wacc, const ComplexParts* cx, cudaStream_t st) {
   using C = Cfg<H>;
   constexpr int TN = C::TN;
+  const int64_t batches = cx ? 2 * p.n_q : p.n_q;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, a, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, kpad, p.M, p.n_q, P4, KSTAGE, TM, P4) ||
-      !make_map(&mb, bop, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, kpad, p.N, p.n_q, P4, KSTAGE, HN, P4))
+  if (!make_map(&ma, a, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, kpad, p.M, batches, P4, KSTAGE, TM, P4) ||
+      !make_map(&mb, bop, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, kpad, p.N, batches, P4, KSTAGE, HN, P4))
     return cudaErrorInvalidValue;
   Tc10Args args;
   args.p = p;
@@ -474,6 +482,12 @@ cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, cons
   args.wacc = wacc;
   args.wrow = tab.wrow;
   args.wcol = tab.wcol;
+  args.parts = cx ? 2 : 1;
+  args.upart = cx ? cx->upart : 0;
+  for (int j = 0; j < 2; ++j) {
+    args.woff[j] = cx ? cx->woff[j] : 0;
+    args.neg[j] = cx ? cx->neg[j] : p.negate;
+  }
   auto kern = gemm_tc10_kernel<H, GEN>;
   thread_local bool attr_set[64] = {};
   int dev = 0;
@@ -484,9 +498,10 @@ cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, cons
     attr_set[dev] = true;
   }
   const int64_t gx = (p.N + TN - 1) / TN, gy = (p.M + TM - 1) / TM;
-  if (gx > 0x7FFFFFFF || gy > 65535 || (int64_t)p.n_q * args.ksplit > 65535) return cudaErrorInvalidConfiguration;
+  const int64_t gz = (int64_t)args.parts * p.n_q * args.ksplit;
+  if (gx > 0x7FFFFFFF || gy > 65535 || gz > 65535) return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)gx, (unsigned)gy, (unsigned)(p.n_q * args.ksplit));
+  cfg.gridDim = dim3((unsigned)gx, (unsigned)gy, (unsigned)gz);
   cfg.blockDim = dim3(C::NTHREADS);
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = st;
@@ -498,23 +513,29 @@ cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, cons
   cudaError_t le = cudaLaunchKernelEx(&cfg, kern, ma, mb, args);
   ++g_kernel_launches;
   if (le != cudaSuccess || args.ksplit == 1) return le;
-  return launch_splitk_round(p, wacc, eu, ev, tab.wrow, tab.wcol, w, err, st);
+  for (int j = 0; j < args.parts && le == cudaSuccess; ++j) {
+    Problem pj = p;
+    pj.negate = args.neg[j];
+    le = launch_splitk_round(pj, wacc + (int64_t)j * p.n_q * p.M * p.N, eu + (int64_t)args.upart * p.n_q * p.M,
+                             ev + (int64_t)j * p.n_q * p.N, tab.wrow, tab.wcol, w + args.woff[j], err, st);
+  }
+  return le;
 }
 
 template <int H>
 cudaError_t launch_tile(const Problem& p, const Tables& tab, const void* a, const void* bop, const int32_t* eu,
                         const int32_t* ev, int64_t kpad, double* w, unsigned* err, int ksplit,
-                        unsigned long long* wacc, cudaStream_t st) {
+                        unsigned long long* wacc, const ComplexParts* cx, cudaStream_t st) {
   if (p.es == 1 && !p.negate && !p.accumulate)
-    return launch_mode<H, false>(p, tab, a, bop, eu, ev, kpad, w, err, ksplit, wacc, st);
-  return launch_mode<H, true>(p, tab, a, bop, eu, ev, kpad, w, err, ksplit, wacc, st);
+    return launch_mode<H, false>(p, tab, a, bop, eu, ev, kpad, w, err, ksplit, wacc, cx, st);
+  return launch_mode<H, true>(p, tab, a, bop, eu, ev, kpad, w, err, ksplit, wacc, cx, st);
 }
 
 }  // namespace
 
 cudaError_t launch_gemm_split10(const Problem& p, const Tables& tab, const uint16_t* us, const uint16_t* vs,
                                 const int32_t* eu, const int32_t* ev, int64_t kpad, double* w, unsigned* err,
-                                int ksplit, unsigned long long* wacc, cudaStream_t st) {
+                                int ksplit, unsigned long long* wacc, const ComplexParts* cx, cudaStream_t st) {
   // The narrower tile where it takes fewer rounds of the SMs.  Clocks measured
   // per stage and per tile: 1930 and 17000 for a 128 x 128 tile, 2270 and 20000
   // for two 128 x 64 tiles side by side (they load the A digits twice: 4650
@@ -522,13 +543,13 @@ cudaError_t launch_gemm_split10(const Problem& p, const Tables& tab, const uint1
   // wide or 264 narrow tiles, takes 103 us instead of 129, preparation included).
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t split = ksplit < 1 ? 1 : ksplit, blocks = ((p.M + TM - 1) / TM) * p.n_q * split;
+  const int64_t split = ksplit < 1 ? 1 : ksplit, blocks = ((p.M + TM - 1) / TM) * p.n_q * split * (cx ? 2 : 1);
   const int64_t n_kb = (kpad / KSTAGE + split - 1) / split;
   const int64_t wide = blocks * ((p.N + 2 * HN - 1) / (2 * HN)), narrow = blocks * ((p.N + HN - 1) / HN);
   const double t2 = (double)((wide + sms - 1) / sms) * (1930.0 * n_kb + 17000.0);
   const double t1 = (double)((narrow + 2 * sms - 1) / (2 * sms)) * (2270.0 * n_kb + 20000.0);
-  if (t1 < 0.9 * t2) return launch_tile<1>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
-  return launch_tile<2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, st);
+  if (t1 < 0.9 * t2) return launch_tile<1>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, cx, st);
+  return launch_tile<2>(p, tab, us, vs, eu, ev, kpad, w, err, ksplit, wacc, cx, st);
 }
 
 }  // namespace symctr

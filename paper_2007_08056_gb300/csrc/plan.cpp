@@ -1119,7 +1119,7 @@ symctr_status run_contract_body(const symctr_plan* P, const double* u, const dou
     const bool two_phase = !skip[0] || !skip[1] || !(rt[0] || rt[1]);
     if (two_phase) {
       e = launch_prep(pc, tab, split, P->n_slices, u, v, base + L.off_a, base + L.off_b, ea, eb, part,
-                      P->kpad, err, barrier, acc, acc_n, skip, st);
+                      P->kpad, err, barrier, acc, acc_n, skip, 1, st);
       if (e != cudaSuccess) return cuda_status(e, "operand preparation");
     }
     if (rt[0] || rt[1]) {
@@ -1288,6 +1288,80 @@ static bool chain_sides(const symctr_plan* src, const std::vector<int>& rows,
   if (in_rows && in_cols) return false;
   (in_cols ? cc : cr)->batch = true;
   return true;
+}
+
+// Complex contraction in the default split form with the digits of all four
+// parts in the workspace at once: each part prepared once (not once for each of
+// the two products it enters) and two GEMM launches of twice the tiles instead
+// of four.  Returns false when the workspace is too small or the plan does not
+// run this form; the caller then takes the parts one product at a time.
+static bool complex_layout(const symctr_plan* P, uint64_t ws_bytes, Layout* L, int64_t* acc_n) {
+  if (!P->tensor_core || P->prec != SYMCTR_SPLIT_BF16 || P->n_slices != 5) return false;
+  Problem both = P->run;
+  both.n_q *= 2;   // real and imaginary parts as batches
+  *L = make_layout(both, true, P->general, P->prec, P->n_slices, P->kpad);
+  // the split-K sums of the second launch follow the first's; then the partial
+  // row maxima of one part's exponent scan
+  *acc_n = L->ksplit > 1 ? 2 * (int64_t)both.n_q * both.M * both.N : 0;
+  L->off_part = (uint64_t)round_up((int64_t)L->bytes + *acc_n / 2 * 8, 256);
+  L->bytes = L->off_part + (uint64_t)prep_partials_entries(P->run) * 4;
+  return L->ok && L->bytes <= ws_bytes;
+}
+
+static symctr_status run_complex_split(const symctr_plan* P, int su, int sv, const double* u, const double* v,
+                                       double* w, void* ws, const Layout& L, int64_t acc_n, cudaStream_t st) {
+  Problem pr = P->run;
+  pr.es = 2;
+  char* base = (char*)ws;
+  unsigned* err = (unsigned*)base;
+  const long long launches0 = g_kernel_launches;
+  cudaError_t e = cudaMemsetAsync(err, 0, 128, st);
+  if (e != cudaSuccess) return cuda_status(e, "clear workspace header");
+  if (P->fill_all || (int64_t)pr.n_q * pr.M * pr.N < P->numel_w) {
+    e = launch_fill_zero(w, 2 * P->numel_w, st);
+    if (e != cudaSuccess) return cuda_status(e, "zero fill");
+  }
+  if (P->prof) cudaEventRecord(P->ev[0], st);
+  const bool attached = tables_attached(P);
+  if (!attached && !P->htab.empty()) pin_tables(P);
+  Tables tab;
+  symctr_status s = pass_tables(P, pr, 0, attached, base, L.off_tab, st, &tab);
+  if (s != SYMCTR_OK) return s;
+  unsigned* barrier = (unsigned*)(base + 64);
+  unsigned long long* acc = acc_n ? (unsigned long long*)(base + L.off_acc) : nullptr;
+  int32_t* ea = (int32_t*)(base + L.off_ea);
+  int32_t* eb = (int32_t*)(base + L.off_eb);
+  int32_t* part = (int32_t*)(base + L.off_part);
+  const int64_t na = (int64_t)pr.n_q * pr.M, nb = (int64_t)pr.n_q * pr.N;
+  for (int j = 0; j < 2; ++j) {
+    if (j == 1) {
+      e = cudaMemsetAsync(barrier, 0, 64, st);
+      if (e != cudaSuccess) return cuda_status(e, "clear barrier");
+    }
+    e = launch_prep(pr, tab, true, P->n_slices, u + j, v + j, base + L.off_a + j * na * P->kpad * 2,
+                    base + L.off_b + j * nb * P->kpad * 2, ea + j * na, eb + j * nb, part, P->kpad, err, barrier,
+                    j == 0 ? acc : nullptr, j == 0 ? acc_n : 0, nullptr, 2, st);
+    if (e != cudaSuccess) return cuda_status(e, "operand preparation");
+  }
+  if (P->prof) cudaEventRecord(P->ev[1], st);
+  // (Ur + i su Ui)(Vr + i sv Vi): U's real part into both parts of W, then its
+  // imaginary part added
+  for (int j = 0; j < 2; ++j) {
+    ComplexParts cx;
+    cx.upart = j;
+    cx.woff[0] = j;
+    cx.woff[1] = 1 - j;
+    cx.neg[0] = j == 1 && su < 0;
+    cx.neg[1] = j == 0 ? sv < 0 : su * sv > 0;
+    pr.accumulate = j;
+    e = launch_gemm_split10(pr, tab, (const uint16_t*)(base + L.off_a), (const uint16_t*)(base + L.off_b), ea, eb,
+                            P->kpad, w, err, L.ksplit, acc ? acc + j * (acc_n / 2) : nullptr, &cx, st);
+    if (e != cudaSuccess) return cuda_status(e, "gemm_split");
+  }
+  if (P->prof) cudaEventRecord(P->ev[2], st);
+  P->last_launches = (int)(g_kernel_launches - launches0);
+  if (!attached && P->pinned) return mark_table_use(P, st);
+  return SYMCTR_OK;
 }
 
 extern "C" {
@@ -1487,6 +1561,10 @@ symctr_status symctr_contract_complex(const symctr_plan* P, int conj_u, int conj
   if (!w || !u || !v) return fail(SYMCTR_ERR_NULLPTR, "NULL tensor pointer");
   cudaStream_t st = (cudaStream_t)stream;
   const double su = conj_u ? -1.0 : 1.0, sv = conj_v ? -1.0 : 1.0;
+  Layout both;
+  int64_t acc_n = 0;
+  if (ws && P->run.n_q > 0 && complex_layout(P, ws_bytes, &both, &acc_n))
+    return run_complex_split(P, su < 0 ? -1 : 1, sv < 0 ? -1 : 1, u, v, w, ws, both, acc_n, st);
   // (Ur + i su Ui)(Vr + i sv Vi) = Ur Vr - su sv Ui Vi + i (sv Ur Vi + su Ui Vr):
   // four real contractions on the real (+0) and imaginary (+1) parts
   struct Term {

@@ -189,18 +189,25 @@ struct Problem {
 // XOR in inline PTX.  Written in C++, the conditional XOR may be folded into a
 // float64 negation, which GB300 issues on its narrow float64 pipe for every
 // stored value.
-__device__ __forceinline__ double signed_result(const Problem& p, double x) {
+template <typename Mode>
+__device__ __forceinline__ double signed_result(const Mode& p, double x) {
   const unsigned mask = p.negate ? 0x80000000u : 0u;
   unsigned hi = (unsigned)__double2hiint(x);
   asm("xor.b32 %0, %0, %1;" : "+r"(hi) : "r"(mask));
   return __hiloint2double((int)hi, __double2loint(x));
 }
 
-// Store of one result into W under the problem's output mode.  The
+// How results enter W: with their sign flipped, added to what is there.
+struct OutMode {
+  int negate, accumulate;
+};
+
+// Store of one result into W under an output mode (a Problem or OutMode).  The
 // accumulating store is a float64 atomic add (performed in L2, each entry
 // with a single writer: the same rounded sum), so that neither mode puts a
 // float64 add on the narrow float64 pipe.
-__device__ __forceinline__ void store_w(const Problem& p, double* dst, double x) {
+template <typename Mode>
+__device__ __forceinline__ void store_w(const Mode& p, double* dst, double x) {
   x = signed_result(p, x);
   if (p.accumulate)
     atomicAdd(dst, x);
@@ -276,12 +283,13 @@ cudaError_t launch_gemm_f64(const Problem& p, const double* u, const double* v, 
                             const Tables* tables, cudaStream_t st);
 cudaError_t launch_fill_zero(double* w, int64_t n, cudaStream_t st);
 // skip[op]: operand op is prepared by launch_rowstream or launch_rowtile
-// instead (NULL: neither)
+// instead (NULL: neither); batch_sets: the digit planes are batch_sets * n_q
+// batches apart (2: ua, va, eu and ev point to the real or the imaginary set)
 cudaError_t launch_prep(const Problem& p, const Tables& t, bool split, int n_slices,
                         const double* u, const double* v, void* ua, void* va, int32_t* eu,
                         int32_t* ev, int32_t* partials, int64_t kpad, unsigned* err, unsigned* barrier,
                         unsigned long long* zero64, int64_t zero64_n, const bool* skip,
-                        cudaStream_t st);
+                        int batch_sets, cudaStream_t st);
 // Single-read split-form preparation of operand op (0 = U, 1 = V) whose
 // aligned rows are runs of `run` contiguous reduced-form entries and at most
 // kRowClusterMaxK long (plan-time eligibility: row_run in plan.cpp); rows
@@ -310,9 +318,16 @@ cudaError_t launch_gemm_split(const Problem& p, const Tables& t, int n_slices, c
                               const uint16_t* vs, const int32_t* eu, const int32_t* ev,
                               int64_t kpad, double* w, unsigned* err, int ksplit,
                               unsigned long long* wacc, cudaStream_t st);
+// Complex products on digits of both parts (2 n_q batches: real, imaginary):
+// part upart of U by both parts of V, part j of V into w + woff[j], negated
+// where neg[j] (the split-K sums of part j follow those of part 0 in wacc).
+struct ComplexParts {
+  int upart;
+  int woff[2], neg[2];
+};
 cudaError_t launch_gemm_split10(const Problem& p, const Tables& t, const uint16_t* us, const uint16_t* vs,
                                 const int32_t* eu, const int32_t* ev, int64_t kpad, double* w,
-                                unsigned* err, int ksplit, unsigned long long* wacc,
+                                unsigned* err, int ksplit, unsigned long long* wacc, const ComplexParts* cx,
                                 cudaStream_t st);
 cudaError_t launch_gemm_tf32(const Problem& p, const Tables& t, const float* u, const float* v,
                              int64_t kpad, double* w, unsigned* err, cudaStream_t st);

@@ -254,6 +254,7 @@ struct PrepArgs {
   unsigned long long* zero64;  // split-K partial sums, zeroed here
   int64_t zero64_n;
   bool skip[2];              // operands prepared by the single-read kernel instead
+  int batch_sets;            // digit planes are batch_sets * n_q batches apart
 };
 
 __device__ __forceinline__ void operand_dims(const Problem& p, int op, int64_t* R, int64_t* Cn) {
@@ -526,7 +527,7 @@ __device__ void slice_unit(const PrepArgs& a, int op, uint32_t unit, int64_t* ro
   const uint32_t b = unit / (rt * ct);
   const uint32_t rem = unit - b * rt * ct;
   const int64_t r0 = (int64_t)(rem / ct) * TILE, cu = (int64_t)(rem % ct) * UCOLS;
-  const int64_t slice_stride = (int64_t)p.n_q * R * kpad;   // elements
+  const int64_t slice_stride = (int64_t)a.batch_sets * p.n_q * R * kpad;   // elements
   const int64_t brow = (int64_t)b * R;
   __syncthreads();
   if (threadIdx.x < TILE) {
@@ -1523,7 +1524,7 @@ cudaError_t launch_rowstream(const Problem& p, const Tables& t, int op, int n_sl
 cudaError_t launch_prep(const Problem& p, const Tables& t, bool split, int n_slices,
                         const double* u, const double* v, void* ua, void* va, int32_t* eu,
                         int32_t* ev, int32_t* partials, int64_t kpad, unsigned* err, unsigned* barrier,
-                        unsigned long long* zero64, int64_t zero64_n, const bool* skip,
+                        unsigned long long* zero64, int64_t zero64_n, const bool* skip, int batch_sets,
                         cudaStream_t st) {
   const int S = split ? n_slices : 0;
   if (S < 0 || S > kMaxSlices) return cudaErrorInvalidValue;
@@ -1589,6 +1590,7 @@ cudaError_t launch_prep(const Problem& p, const Tables& t, bool split, int n_sli
   a.zero64_n = zero64_n;
   a.skip[0] = skip && skip[0];
   a.skip[1] = skip && skip[1];
+  a.batch_sets = batch_sets;
   void* params[] = {&a};
   cudaError_t e = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(THREADS),
                                               params, 0, st);

@@ -86,3 +86,31 @@ def test_mps_transfer_with_conjugate(sc, precision):
     o2 = O.plan(WL.MPS_STEP2, G, o1.sym_w, O.Sym(*negated(sA)))
     want = O.contract_blockloop(o2, Xr, np.conj(A))
     assert rel(Ep.cpu().numpy(), want) <= TOL[precision]
+
+
+@pytest.mark.parametrize("conj", [(False, False), (True, True), (False, True)], ids=["UV", "cU-cV", "U-cV"])
+@pytest.mark.parametrize("dims", [(3, 40, 2), (8, 64, 2), (2, 9, 1), (5, 33, 3)], ids=str)
+def test_both_parts_at_once(sc, dims, conj):
+    """The default split form with both parts' digits in the workspace (split and
+    whole K ranges, half tiles, an output with entries no irrep writes), and with
+    a workspace that holds one part only: the parts one product at a time."""
+    G, bond, phys = dims
+    cu, cv = conj
+    for es, su, sv in [("ab,asg->bsg", ((1, -1), (0,), (bond, bond)), ((1, 1, -1), (1,), (bond, phys, bond))),
+                       ("bsg,bsd->gd", ((1, 1, -1), (0,), (bond, phys, bond)), ((1, 1, -1), (0,), (bond, phys, bond))),
+                       ("ab,cb->ac", ((1, -1), (0,), (bond, 8)), ((1, -1), (0,), (bond + 3, 8)))]:
+        u, v = cdraw((G,), su, 31), cdraw((G,), sv, 32)
+        v = v * (1.0 + 1e-6j)
+        pu, pv = (negated(su) if cu else su), (negated(sv) if cv else sv)
+        p = sc.Plan(es, (G,), pu, pv, "split_bf16")
+        ud, vd = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+        o = O.plan(es, O.Group((G,)), O.Sym(*pu), O.Sym(*pv))
+        want = O.contract_blockloop(o, np.conj(u) if cu else u, np.conj(v) if cv else v)
+        small = torch.empty(int(p.info.workspace_bytes), dtype=torch.uint8, device="cuda")
+        for ws in (None, small):
+            w = p.contract_complex(ud, vd, conj_u=cu, conj_v=cv, workspace=ws,
+                                   out=torch.full(p.shape_w, np.nan, dtype=torch.complex128, device="cuda"))
+            torch.cuda.synchronize()
+            p.check_device_error(ws)
+            assert rel(w.cpu().numpy().real, want.real) <= TOL["split_bf16"]
+            assert rel(w.cpu().numpy().imag, want.imag) <= TOL["split_bf16"]
