@@ -46,9 +46,7 @@ cudaError_t launch_fill_dead(double* w, int64_t bv, int64_t n_combo, const uint3
   FillMask m{};
   for (int64_t k = 0; k < (n_combo + 31) / 32; ++k) m.bits[k] = written[k];
   const int64_t chunks = (bv + kFillChunk - 1) / kFillChunk, items = n_combo * chunks;
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t cap = (int64_t)sms * 8;
+  const int64_t cap = (int64_t)device_sms() * 8;
   fill_dead_kernel<<<(int)(items < cap ? items : cap), kFillThreads, 0, st>>>(w, bv, chunks, items, m);
   ++g_kernel_launches;
   return cudaGetLastError();

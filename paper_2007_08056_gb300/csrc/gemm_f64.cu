@@ -613,12 +613,6 @@ __global__ void __launch_bounds__(THREADS, 4)
   }
 }
 
-int sm_count() {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 // Zero the entries of W that a split-K launch accumulates into.
 __global__ void zero_w_entries(const __grid_constant__ Problem p, double* __restrict__ W) {
   int64_t total = (int64_t)p.n_q * p.M * p.N;
@@ -734,7 +728,7 @@ TileChoice tile_choice(const Problem& p, int sms) {
 cudaError_t launch_gemm_f64(const Problem& p, const double* u, const double* v, double* w,
                             const Tables* tables, cudaStream_t st) {
   if (p.n_q == 0 || p.M == 0 || p.N == 0) return cudaSuccess;
-  const int sms = sm_count();
+  const int sms = device_sms();
   // general plans take the tiled kernel with their tables (every shape)
   bool skinny = !tables && (p.M < 16 || p.N < 16);
   if (skinny && (p.M <= SKINNY_MAX || p.N <= SKINNY_MAX)) {

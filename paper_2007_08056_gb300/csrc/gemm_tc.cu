@@ -766,8 +766,7 @@ cudaError_t launch_splitk_round(const Problem& p, const unsigned long long* wacc
                                 const unsigned* err, cudaStream_t st) {
   // one thread per kRoundRows outputs
   const int64_t work = (int64_t)p.n_q * ((p.M + kRoundRows - 1) / kRoundRows) * p.N;
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int64_t blocks = (work + kRoundThreads - 1) / kRoundThreads;
   cudaLaunchConfig_t rc = {};
   rc.gridDim = dim3((unsigned)(blocks < (int64_t)sms * 8 ? blocks : (int64_t)sms * 8));

@@ -541,8 +541,7 @@ cudaError_t launch_gemm_split10(const Problem& p, const Tables& tab, const uint1
   // for two 128 x 64 tiles side by side (they load the A digits twice: 4650
   // against 4100 us for the CC ladder, but 1285 x 192 x 738 by 8 irreps, 176
   // wide or 264 narrow tiles, takes 103 us instead of 129, preparation included).
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int64_t split = ksplit < 1 ? 1 : ksplit, blocks = ((p.M + TM - 1) / TM) * p.n_q * split * (cx ? 2 : 1);
   const int64_t n_kb = (kpad / KSTAGE + split - 1) / split;
   const int64_t wide = blocks * ((p.N + 2 * HN - 1) / (2 * HN)), narrow = blocks * ((p.N + HN - 1) / HN);

@@ -275,6 +275,17 @@ constexpr int kKChunk = 64;         // K between exact flushes of the top accumu
 // Kernels launched on this host thread (every launcher adds its launches).
 extern thread_local long long g_kernel_launches;
 
+// SMs of the current device, asked once per host thread and device.
+inline int device_sms() {
+  thread_local int cache[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  if (cache[dev] == 0 && (cudaDeviceGetAttribute(&cache[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+                          cache[dev] < 1))
+    cache[dev] = 148;
+  return cache[dev];
+}
+
 // ---- kernel launchers (return cudaError_t of the launch) ----
 // `tables` (general plans only, else NULL): the offset tables of all batches.
 cudaError_t launch_align_f64(const Problem& p, int operand, int direction, const double* src,

@@ -707,7 +707,10 @@ __global__ void __launch_bounds__(THREADS, 4) prep_kernel(PrepArgs a) {
 // unit-stride layout) and fits in shared memory, one CTA per SM instead
 // streams whole rows into shared memory with bulk copies (one per run, on an
 // mbarrier, up to kRsMaxBufs rows in flight), takes the row maximum there and writes
-// the row's digits from there: every operand entry crosses HBM once.
+// the row's digits from there: every operand entry crosses HBM once.  Rows of up
+// to 4096 entries go to two CTAs per SM with three rows each: the barriers and
+// reductions of a row, a third of its time at that length, overlap (4096 x 4096
+// by 16 irreps 1031 -> 790 us).
 // ---------------------------------------------------------------------------
 constexpr int RS_THREADS = 512;
 constexpr int kRsMaxBufs = 6;          // rows in flight per CTA (as shared memory allows)
@@ -812,8 +815,8 @@ __device__ __forceinline__ int rs_row_k0(const RowStreamArgs& a, const double* r
 // rows earlier), then one barrier frees row i's buffer for its refill and
 // publishes row i + 1's maximum.  The maxima rotate over three shared words,
 // each cleared two barriers before its next use.
-template <int S>
-__global__ void __launch_bounds__(RS_THREADS, 1) rowstream_kernel(const __grid_constant__ RowStreamArgs a) {
+template <int S, int PER_SM>
+__global__ void __launch_bounds__(RS_THREADS, PER_SM) rowstream_kernel(const __grid_constant__ RowStreamArgs a) {
   extern __shared__ __align__(128) uint8_t rs_smem[];
   __shared__ __align__(8) uint64_t bars[kRsMaxBufs];
   __shared__ unsigned long long red[RS_THREADS / 32];
@@ -1135,9 +1138,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) rowcluster_kernel(const __grid_
 }
 
 int grid_for(int64_t tiles) {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int64_t cap = (int64_t)sms * 8;
+  int64_t cap = (int64_t)device_sms() * 8;
   return (int)(tiles < cap ? (tiles > 0 ? tiles : 1) : cap);
 }
 
@@ -1159,9 +1160,18 @@ void operand_extent(const Problem& p, int operand, int64_t* R, int64_t* Cn) {
 // there and writes the row's digits from there.  No grid barrier: the
 // operands' preparation is one plain launch.
 // ---------------------------------------------------------------------------
-constexpr int RT_THREADS = 512;
+// Threads of a CTA: 512, two CTAs to an SM, while every unit has an SM nearly to
+// itself (the latency of one unit counts); 256, four CTAs, beyond kRtManyUnits
+// units per SM, so that one CTA's copies run beside another's digits
+// (40960 x 640 x 640 by 10 irreps: 4.26 -> 4.00 ms with the contraction; the MPS
+// step 73 -> 75 us, hence the rule).
+constexpr int kRtManyUnits = 12;
 
 // 8-byte asynchronous copy global -> shared; src_bytes 0 fills zeros (reads nothing)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async8(void* dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
                : "memory");
@@ -1177,14 +1187,15 @@ struct RowTileArgs {
   uint32_t* dst[2];          // BF16 digit pairs: [S][n_q][R][kpad / 2]
   int32_t* exps[2];          // [n_q][R] biased row exponents
   bool fast_rows[2];
+  bool pair_ok[2];           // column-contiguous with every offset of an even column even
   size_t buf_off;            // byte offset of the row buffer in shared memory
   unsigned* err;
   unsigned long long* zero64;  // split-K partial sums, zeroed here
   int64_t zero64_n;
 };
 
-template <int S>
-__global__ void __launch_bounds__(RT_THREADS) rowtile_kernel(const __grid_constant__ RowTileArgs a) {
+template <int S, int RT_THREADS>
+__global__ void __launch_bounds__(RT_THREADS, 1024 / RT_THREADS) rowtile_kernel(const __grid_constant__ RowTileArgs a) {
   extern __shared__ __align__(16) uint8_t rt_smem[];
   const Problem& p = a.p;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1246,6 +1257,16 @@ __global__ void __launch_bounds__(RT_THREADS) rowtile_kernel(const __grid_consta
         const int64_t co = coff[k];
         const bool ok = ro >= 0 && co >= 0;
         cp_async8(brow + k, ok ? rowp + co : src, ok ? 8u : 0u);
+      }
+    } else if (a.pair_ok[op]) {
+      // lanes on consecutive column pairs, one 16-byte copy each
+      for (int r = warp / wpr; r < R; r += NW / wpr) {
+        const int64_t ro = roff[r];
+        const double* rowp = src + (ro >= 0 ? ro : 0);
+        double* brow = buf + r * LD;
+#pragma unroll 4
+        for (int k = 2 * (sub * 32 + lane); k < Kc; k += 64 * wpr)
+          cp_async16(brow + k, rowp + coff[k], ro >= 0 ? 16u : 0u);
       }
     } else {
       // lanes on consecutive columns, wpr warps per row
@@ -1341,15 +1362,6 @@ cudaError_t launch_rowtile(const Problem& p, const Tables& t, int n_slices, cons
   if (n_slices < 1 || n_slices > kMaxSlices || p.es != 1 || p.K < 1 || kpad > kRowTileMaxK ||
       kpad % 32 != 0 || kpad < p.K)
     return cudaErrorInvalidValue;
-  void (*kern)(RowTileArgs) = nullptr;
-  switch (n_slices) {
-    case 1: kern = rowtile_kernel<1>; break;
-    case 2: kern = rowtile_kernel<2>; break;
-    case 3: kern = rowtile_kernel<3>; break;
-    case 4: kern = rowtile_kernel<4>; break;
-    case 5: kern = rowtile_kernel<5>; break;
-    default: kern = rowtile_kernel<6>; break;
-  }
   RowTileArgs a;
   a.p = p;
   a.t = t;
@@ -1369,6 +1381,9 @@ cudaError_t launch_rowtile(const Problem& p, const Tables& t, int n_slices, cons
   a.exps[1] = ev;
   a.fast_rows[0] = rows_fast(p.u);
   a.fast_rows[1] = rows_fast(p.v);
+  // (16-byte aligned operands; the columns of a pair exist together)
+  a.pair_ok[0] = !p.general && !a.fast_rows[0] && pairs_aligned(p.u) && ((uintptr_t)u & 15) == 0;
+  a.pair_ok[1] = !p.general && !a.fast_rows[1] && pairs_aligned(p.v) && ((uintptr_t)v & 15) == 0;
   a.buf_off = rowtile_head_bytes(p.K, R);
   a.err = err;
   a.zero64 = zero64;
@@ -1378,32 +1393,43 @@ cudaError_t launch_rowtile(const Problem& p, const Tables& t, int n_slices, cons
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 16) return cudaErrorInvalidDevice;
+  const int sms = device_sms();
+  const int many = units[0] + units[1] > (int64_t)kRtManyUnits * sms ? 1 : 0;
+  const int threads = many ? 256 : 512;
+  void (*kern)(RowTileArgs) = nullptr;
+  switch (n_slices) {
+    case 1: kern = many ? rowtile_kernel<1, 256> : rowtile_kernel<1, 512>; break;
+    case 2: kern = many ? rowtile_kernel<2, 256> : rowtile_kernel<2, 512>; break;
+    case 3: kern = many ? rowtile_kernel<3, 256> : rowtile_kernel<3, 512>; break;
+    case 4: kern = many ? rowtile_kernel<4, 256> : rowtile_kernel<4, 512>; break;
+    case 5: kern = many ? rowtile_kernel<5, 256> : rowtile_kernel<5, 512>; break;
+    default: kern = many ? rowtile_kernel<6, 256> : rowtile_kernel<6, 512>; break;
+  }
   // The shared-memory attribute belongs to the function, not to the host
   // thread: every thread sets the same value, the most any row length needs,
   // so that no thread lowers what another one relies on.
-  thread_local bool attr_set[kMaxSlices + 1][16] = {};
-  if (!attr_set[n_slices][dev]) {
+  thread_local bool attr_set[2][kMaxSlices + 1][16] = {};
+  if (!attr_set[many][n_slices][dev]) {
     e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)rowtile_smem_bytes(kRowTileMaxK, kRowTileMaxK));
     if (e != cudaSuccess) return e;
-    attr_set[n_slices][dev] = true;
+    attr_set[many][n_slices][dev] = true;
   }
   // resident CTAs at this call's shared memory, kept for the size last asked
-  thread_local size_t resident_smem[kMaxSlices + 1][16] = {};
-  thread_local int resident[kMaxSlices + 1][16] = {};
-  if (resident_smem[n_slices][dev] != smem) {
-    int sms = 0, per = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, RT_THREADS, smem);
+  thread_local size_t resident_smem[2][kMaxSlices + 1][16] = {};
+  thread_local int resident[2][kMaxSlices + 1][16] = {};
+  if (resident_smem[many][n_slices][dev] != smem) {
+    int per = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem);
     if (e != cudaSuccess) return e;
-    resident[n_slices][dev] = sms * (per > 0 ? per : 1);
-    resident_smem[n_slices][dev] = smem;
+    resident[many][n_slices][dev] = sms * (per > 0 ? per : 1);
+    resident_smem[many][n_slices][dev] = smem;
   }
   const int64_t work = units[0] + units[1];
-  const int64_t zero_ctas = (zero64_n + RT_THREADS - 1) / RT_THREADS;
+  const int64_t zero_ctas = (zero64_n + threads - 1) / threads;
   int64_t grid = work > 0 ? work : (zero_ctas > 0 ? zero_ctas : 1);
-  if (grid > resident[n_slices][dev]) grid = resident[n_slices][dev];
-  kern<<<(unsigned)grid, RT_THREADS, smem, st>>>(a);
+  if (grid > resident[many][n_slices][dev]) grid = resident[many][n_slices][dev];
+  kern<<<(unsigned)grid, threads, smem, st>>>(a);
   ++g_kernel_launches;
   return cudaGetLastError();
 }
@@ -1441,33 +1467,33 @@ cudaError_t launch_rowstream(const Problem& p, const Tables& t, int op, int n_sl
   // [r seg, (r+1) seg) (seg a multiple of 4, so every piece of a run stays even)
   const int C = (int)((K + kRowStreamMaxK - 1) / kRowStreamMaxK);
   const int64_t seg = C > 1 ? ((K + C - 1) / C + 3) / 4 * 4 : K;
+  // rows of at most 32 KB: two CTAs per SM with three rows each
+  const size_t row_bytes = (size_t)((seg + 15) / 16 * 16) * sizeof(double);
+  const int form = C > 1 ? 2 : 3 * row_bytes <= kRsSmem / 2 ? 1 : 0;
   void (*kern)(RowStreamArgs) = nullptr;
   switch (n_slices) {
-    case 2: kern = C > 1 ? rowcluster_kernel<2> : rowstream_kernel<2>; break;
-    case 3: kern = C > 1 ? rowcluster_kernel<3> : rowstream_kernel<3>; break;
-    case 4: kern = C > 1 ? rowcluster_kernel<4> : rowstream_kernel<4>; break;
-    case 5: kern = C > 1 ? rowcluster_kernel<5> : rowstream_kernel<5>; break;
-    default: kern = C > 1 ? rowcluster_kernel<6> : rowstream_kernel<6>; break;
+    case 2: kern = form == 2 ? rowcluster_kernel<2> : form == 1 ? rowstream_kernel<2, 2> : rowstream_kernel<2, 1>; break;
+    case 3: kern = form == 2 ? rowcluster_kernel<3> : form == 1 ? rowstream_kernel<3, 2> : rowstream_kernel<3, 1>; break;
+    case 4: kern = form == 2 ? rowcluster_kernel<4> : form == 1 ? rowstream_kernel<4, 2> : rowstream_kernel<4, 1>; break;
+    case 5: kern = form == 2 ? rowcluster_kernel<5> : form == 1 ? rowstream_kernel<5, 2> : rowstream_kernel<5, 1>; break;
+    default: kern = form == 2 ? rowcluster_kernel<6> : form == 1 ? rowstream_kernel<6, 2> : rowstream_kernel<6, 1>; break;
   }
-  const size_t row_bytes = (size_t)((seg + 15) / 16 * 16) * sizeof(double);
-  int nbuf = (int)(kRsSmem / row_bytes);
+  int nbuf = (int)((form == 1 ? kRsSmem / 2 : kRsSmem) / row_bytes);
   if (nbuf > kRsMaxBufs) nbuf = kRsMaxBufs;
   if (nbuf < 2) return cudaErrorInvalidValue;
   const size_t smem = (size_t)nbuf * row_bytes;
   // (the attribute belongs to the function: every thread sets the same value)
-  thread_local bool attr_set[2][kMaxSlices + 1][16] = {};
+  thread_local bool attr_set[3][kMaxSlices + 1][16] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 16) return cudaErrorInvalidDevice;
-  if (!attr_set[C > 1][n_slices][dev]) {
+  if (!attr_set[form][n_slices][dev]) {
     e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsSmem);
     if (e != cudaSuccess) return e;
-    attr_set[C > 1][n_slices][dev] = true;
+    attr_set[form][n_slices][dev] = true;
   }
-  int sms = 0;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
+  const int sms = device_sms();
   RowStreamArgs a;
   a.R = R;
   a.K = K;
@@ -1485,7 +1511,8 @@ cudaError_t launch_rowstream(const Problem& p, const Tables& t, int op, int n_sl
   a.seg = seg;
   const int64_t rows = (int64_t)p.n_q * R;
   if (C == 1) {
-    const int grid = (int)(rows < sms ? (rows > 0 ? rows : 1) : sms);
+    const int most = form == 1 ? 2 * sms : sms;
+    const int grid = (int)(rows < most ? (rows > 0 ? rows : 1) : most);
     kern<<<grid, RS_THREADS, smem, st>>>(a);
     ++g_kernel_launches;
     return cudaGetLastError();
