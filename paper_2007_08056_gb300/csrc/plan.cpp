@@ -1113,7 +1113,9 @@ symctr_status run_contract_body(const symctr_plan* P, const double* u, const dou
     const bool rs[2] = {split && pr.es == 1 && P->row_run[0] > 0, split && pr.es == 1 && P->row_run[1] > 0};
     // short rows take the short-row kernel (real data only)
     const bool rt[2] = {split && pr.es == 1 && P->row_tile[0], split && pr.es == 1 && P->row_tile[1]};
-    const bool skip[2] = {rs[0] || rt[0], rs[1] || rt[1]};
+    // TF32: a long operand against a short one is read by the GEMM itself
+    const int direct = split ? -1 : tf32_direct_operand(pc, u, v);
+    const bool skip[2] = {rs[0] || rt[0] || direct == 0, rs[1] || rt[1] || direct == 1};
     // the two-phase kernel runs for an operand left to it, or to zero the
     // split-K sums when no short-row kernel runs
     const bool two_phase = !skip[0] || !skip[1] || !(rt[0] || rt[1]);
@@ -1138,6 +1140,9 @@ symctr_status run_contract_body(const symctr_plan* P, const double* u, const dou
       e = launch_gemm_split(pc, tab, P->n_slices, (const uint16_t*)(base + L.off_a),
                             (const uint16_t*)(base + L.off_b), ea, eb, P->kpad, w, err, L.ksplit,
                             acc, st);
+    else if (direct >= 0)
+      e = launch_gemm_tf32_direct(pc, tab, direct, direct == 0 ? u : v,
+                                  (const float*)(base + (direct == 0 ? L.off_b : L.off_a)), P->kpad, w, err, st);
     else
       e = launch_gemm_tf32(pc, tab, (const float*)(base + L.off_a),
                            (const float*)(base + L.off_b), P->kpad, w, err, st);

@@ -340,6 +340,13 @@ cudaError_t launch_gemm_split10(const Problem& p, const Tables& t, const uint16_
                                 const int32_t* eu, const int32_t* ev, int64_t kpad, double* w,
                                 unsigned* err, int ksplit, unsigned long long* wacc, const ComplexParts* cx,
                                 cudaStream_t st);
+// TF32 product read from operand op's float64 reduced form itself, with the other
+// operand (at most kTf32DirectShort aligned rows) as FP32 rows; the operand that
+// allows it, or -1 (see gemm_tf32_direct.cu, transforms.cu).
+constexpr int64_t kTf32DirectShort = 512;
+int tf32_direct_operand(const Problem& p, const double* u, const double* v);
+cudaError_t launch_gemm_tf32_direct(const Problem& p, const Tables& t, int op, const double* src, const float* other,
+                                    int64_t kpad, double* w, unsigned* err, cudaStream_t st);
 cudaError_t launch_gemm_tf32(const Problem& p, const Tables& t, const float* u, const float* v,
                              int64_t kpad, double* w, unsigned* err, cudaStream_t st);
 

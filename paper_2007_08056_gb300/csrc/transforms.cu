@@ -1548,6 +1548,21 @@ cudaError_t launch_rowstream(const Problem& p, const Tables& t, int op, int n_sl
   return e;
 }
 
+// The TF32 form reads operand op without a copy when its column pairs are 16-byte
+// loads, the other side fits one tile (512 rows), and op is long: at least four
+// times the other side, and 128-row tiles for most SMs.
+int tf32_direct_operand(const Problem& p, const double* u, const double* v) {
+  if (p.es != 1 || p.general || p.negate || p.accumulate || p.n_q > 65535) return -1;
+  for (int op = 0; op < 2; ++op) {
+    const int64_t rows = op == 0 ? p.M : p.N, other = op == 0 ? p.N : p.M;
+    const OperandMap& m = op == 0 ? p.u : p.v;
+    if (other > kTf32DirectShort || rows < 4 * other || (rows + 127) / 128 * p.n_q < 128 || p.K < 64) continue;
+    if (rows_fast(m) || !pairs_aligned(m) || ((uintptr_t)(op == 0 ? u : v) & 15) != 0) continue;
+    return op;
+  }
+  return -1;
+}
+
 cudaError_t launch_prep(const Problem& p, const Tables& t, bool split, int n_slices,
                         const double* u, const double* v, void* ua, void* va, int32_t* eu,
                         int32_t* ev, int32_t* partials, int64_t kpad, unsigned* err, unsigned* barrier,
