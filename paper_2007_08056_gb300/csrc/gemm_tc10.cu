@@ -24,7 +24,9 @@
 // exponents (integer arithmetic only: GB300 has little float64 throughput).
 //
 // CTA: 640 threads: warp 0 TMA, warps 1 and 2 MMA, warps 4-19 drains and
-// epilogue; one 128 x 128 tile, 512 TMEM columns, three stages of 64 KB.  The
+// epilogue; 128 x 128 tiles, 512 TMEM columns, three stages of 64 KB.  The grid is
+// resident as a whole and each CTA walks tiles one grid apart: the next tile's
+// first loads and MMAs run beside the rounding and writing of the last one.  The
 // tile is two halves of 64 columns with their own four accumulators side by
 // side: one MMA per A digit takes all the B digits it pairs with (N = 256, 192,
 // 128, 64).  Each half has its own issuing thread and its own 8 warps, so that
@@ -39,8 +41,11 @@
 // between MMAs, 2650 with both halves issued by one thread, whose waits leave
 // the tensor pipe empty, 2970 for the five BF16 digits before.  Float-to-int
 // conversions run at 16 per clock and SM here, so the drains use magic-number
-// adds (3470 with conversions).  CC ladder step 6.68 -> 5.59 ms, (2,2,2) with
-// D = 23 1.02 -> 0.85 ms, 40960 x 640 x 640 by 10 irreps 5.11 -> 4.44 ms.
+// adds (3470 with conversions).  CC ladder step 6.68 -> 5.49 ms, (2,2,2) with
+// D = 23 1.02 -> 0.81 ms, 40960 x 640 x 640 by 10 irreps 5.11 -> 3.70 ms (3.99
+// with a CTA to a tile, whose setup, first loads and writes nothing covered).
+// The drain loop leaves no register to spare: with 80 bytes of spills instead of
+// 32 that last case takes 4.01 ms.
 // Every wait is bounded (see tc_common.cuh).
 #include "tc_common.cuh"
 
@@ -55,6 +60,10 @@ constexpr int P4 = 4;             // digit planes
 constexpr int ROWB = 64;          // bytes per tile row and stage: 32 FP16, SWIZZLE_64B
 constexpr int KSTAGE = 32;
 constexpr int kFold = 16;         // stages between folds of diagonal 2 (even)
+// Whether diagonal 2 is folded in the drain that has `left` drains behind it (only
+// every second drain folds: the first in a pair asks nothing).  Counted from the
+// end, so that a K range of kFold stages has none.
+__device__ __forceinline__ bool folds_after(int left) { return (left / 2) % (kFold / 2) == kFold / 2 - 1; }
 constexpr int A_BYTES = P4 * TM * ROWB;     // all digits of a stage's A tile
 constexpr int B_BYTES = P4 * HN * ROWB;     // of one half's B tile
 
@@ -66,11 +75,16 @@ struct Cfg {
   static constexpr int NTHREADS = 128 + 32 * EPI_WARPS;
   static constexpr int STAGES = H == 2 ? 3 : 2;
   static constexpr int STAGE_BYTES = A_BYTES + H * B_BYTES;
-  static constexpr int LD = TN + 1;        // epilogue staging stride (doubles)
   static constexpr size_t REGION = (size_t)STAGES * STAGE_BYTES;
-  static_assert(REGION >= (size_t)TM * LD * 8, "the epilogue staging fits the stages");
-  static constexpr int BARS = 2 * STAGES + 6;
-  static constexpr size_t SMEM = 1024 + REGION + 8 * BARS + 12 * (TN + TM) + 16 + 64;
+  // The epilogue staging (TM x TN 64-bit words) overlays the first stages; a tile
+  // starts with stage FIRST, which at H = 2 lies behind it.
+  static constexpr size_t STAGING = (size_t)TM * TN * 8;
+  static_assert(REGION >= STAGING, "the epilogue staging fits the stages");
+  static constexpr int FIRST = STAGES - 1;
+  static constexpr bool EARLY = (size_t)FIRST * STAGE_BYTES >= STAGING;   // loads beside the epilogue
+  static constexpr int BARS = 2 * STAGES + 7;
+  static constexpr int TAB = 12 * (TN + TM);      // offsets and exponents of a tile
+  static constexpr size_t SMEM = REGION + 8 * BARS + 2 * TAB + 16 + 64;
 };
 
 // K-major rows of 64 bytes, SWIZZLE_64B, 8-row groups 512 bytes apart.
@@ -127,53 +141,87 @@ struct Tc10Args {
   // parts * n_q * ksplit), part j into W + woff[j] with sign neg[j].
   int parts, upart;
   int woff[2], neg[2];
+  int gx, gy;        // column and row blocks
+  uint32_t tiles;    // gx * gy * parts * n_q * ksplit
 };
+
+// The thread's index, read again.
+__device__ __forceinline__ int tid_again() {
+  int t;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+  return t;
+}
+
+// Whether `ok` holds for all of the N threads that meet here (named barrier 1).
+template <int N>
+__device__ __forceinline__ bool all_ok(bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+      "barrier.cta.red.and.pred.aligned q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(r)
+      : "r"((uint32_t)ok), "n"(N)
+      : "memory");
+  return r != 0;
+}
 
 template <int H, bool GEN>
 __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
     gemm_tc10_kernel(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b,
                      const __grid_constant__ Tc10Args args) {
   using C = Cfg<H>;
-  constexpr int TN = C::TN, STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, LD = C::LD;
+  constexpr int TN = C::TN, STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES;
   constexpr int EPI_WARPS = C::EPI_WARPS;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  // (alignment by declaration: addresses within are constants, not registers)
+  extern __shared__ __align__(1024) uint8_t smem[];
   const Problem& p = args.p;
-  uint8_t* tiles = smem;  // [STAGES][A digits, B digits of half 0, of half 1], later the epilogue staging
+  uint8_t* tiles = smem;  // [STAGES][A digits, B digits of half 0, of half 1], also the epilogue staging
   uint64_t* full = (uint64_t*)(smem + C::REGION);
   uint64_t* empty = full + STAGES;
   uint64_t* go = empty + STAGES;         // [2] a half's MMAs of a stage are done: drain
   uint64_t* drained = go + 2;            // [2] its accumulators may be written again
-  uint64_t* acc_full = drained + 2;
-  uint64_t* zero_done = acc_full + 1;
-  int64_t* coff = (int64_t*)(zero_done + 1);   // [TN] W column offsets
-  int64_t* roffs = coff + TN;                  // [TM] W row offsets
-  int32_t* cexp = (int32_t*)(roffs + TM);      // [TN] column exponents
-  int32_t* rexps = cexp + TN;                  // [TM] row exponents
-  uint32_t* tmem_slot = (uint32_t*)(rexps + TM);
+  uint64_t* acc_full = drained + 2;      // a tile's MMAs are done
+  uint64_t* zero_done = acc_full + 1;    // its accumulators are read out and zeroed
+  uint64_t* staged = zero_done + 1;      // its results have left the staging
+  uint8_t* tabs = (uint8_t*)(staged + 1);      // [2] tables of this tile and the last one
+  uint32_t* tmem_slot = (uint32_t*)(tabs + 2 * C::TAB);
   Ctl* ctl = (Ctl*)(tmem_slot + 4);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t n0 = (int64_t)blockIdx.x * TN, m0 = (int64_t)blockIdx.y * TM;
-  const int zb = blockIdx.z / args.ksplit;       // part * n_q + irrep
-  const int ks = blockIdx.z % args.ksplit;
-  const int part_v = zb >= p.n_q ? 1 : 0, b = zb - part_v * p.n_q;
-  const int ub = b + args.upart * p.n_q;         // U's batch (V's is zb)
-  const int kb0 = ks * args.kb_per_split;
-  const int n_kb = min(args.n_kb, kb0 + args.kb_per_split) - kb0;
-  const int halves = H == 2 && p.N - n0 > HN ? 2 : 1;
+  // Tile t: column block fastest (its neighbours share the rows of U).
+  struct Tile {
+    int n0, m0;
+    int ub, vb, b, part;      // U's and V's batch, irrep, part of W (complex)
+    int kb0, n_kb, halves;    // K range
+  };
+  auto tile_at = [&](uint32_t t) {
+    Tile x;
+    const uint32_t g = t / (uint32_t)args.gx, z = g / (uint32_t)args.gy;
+    x.n0 = (int)(t - g * (uint32_t)args.gx) * TN;
+    x.m0 = (int)(g - z * (uint32_t)args.gy) * TM;
+    x.vb = (int)(z / (uint32_t)args.ksplit);      // part * n_q + irrep
+    const int ks = (int)z - x.vb * args.ksplit;
+    x.part = x.vb >= p.n_q ? 1 : 0;
+    x.b = x.vb - x.part * p.n_q;
+    x.ub = x.b + args.upart * p.n_q;
+    x.kb0 = ks * args.kb_per_split;
+    x.n_kb = min(args.n_kb, x.kb0 + args.kb_per_split) - x.kb0;
+    x.halves = H == 2 && p.N - x.n0 > HN ? 2 : 1;
+    return x;
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], halves);
+      mbar_init(&empty[s], H);
     }
     for (int h = 0; h < 2; ++h) {
       mbar_init(&go[h], 1);
       mbar_init(&drained[h], 8);
     }
-    mbar_init(acc_full, halves);
-    mbar_init(zero_done, 8 * halves);
+    mbar_init(acc_full, H);
+    mbar_init(zero_done, 8 * H);
+    mbar_init(staged, 8 * H);
     ctl->abort = 0;
     ctl->err = args.err;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -184,19 +232,9 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // W's offset tables are constants of the plan: read before the wait.
-  const int et = (int)threadIdx.x - EPI_WARP0 * 32;   // epilogue thread
-  if (et >= 0 && et < TM) {
-    roffs[et] = m0 + et < p.M ? args.wrow[(int64_t)b * p.M + m0 + et] : -1;
-    if (et < TN) coff[et] = n0 + et < p.N ? args.wcol[(int64_t)b * p.N + n0 + et] : -1;
-  }
   // Launched as a programmatic dependent of the operand preparation: the setup
   // above overlaps its tail; everything below reads its outputs.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (et >= 0 && et < TM) {
-    rexps[et] = m0 + et < p.M ? args.eu[(int64_t)ub * p.M + m0 + et] - kExpBias : 0;
-    if (et < TN) cexp[et] = n0 + et < p.N ? args.ev[(int64_t)zb * p.N + n0 + et] - kExpBias : 0;
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -212,26 +250,39 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
-      int issued = 0;
-      for (int kb = 0; kb < n_kb; ++kb) {
-        const int st = kb % STAGES;
-        if (!wait_phase(&empty[st], ((kb / STAGES) & 1) ^ 1, ctl)) break;
-        mbar_expect_tx(&full[st], A_BYTES + halves * B_BYTES);
-        uint8_t* sa = tiles + (size_t)st * STAGE_BYTES;
-        // all four digit tiles of an operand in one copy
-        const int kc = (kb0 + kb) * KSTAGE;
-        tma_load_4d(&tma_a, &full[st], sa, kc, (int)m0, ub);
-        tma_load_4d(&tma_b, &full[st], sa + A_BYTES, kc, (int)n0, zb);
-        if (halves == 2) tma_load_4d(&tma_b, &full[st], sa + A_BYTES + B_BYTES, kc, (int)n0 + HN, zb);
-        ++issued;
+      uint32_t ph = 0;          // bit s: parity of stage s's next use
+      int n_tile = 0, st = 0;
+      bool ok = true;
+      uint32_t live = 0;        // stages with a copy issued
+      for (uint32_t t = blockIdx.x; ok && t < args.tiles; t += gridDim.x, ++n_tile) {
+        const Tile x = tile_at(t);
+        st = C::FIRST;
+        for (int kb = 0; kb < x.n_kb; ++kb) {
+          // the stages under the last tile's staging wait until it is read out
+          // (one phase a tile, waited for before this tile's last stage is loaded)
+          const int under = C::EARLY && x.n_kb > 1 ? 1 : 0;
+          if (n_tile > 0 && kb == under) ok = wait_phase(staged, (n_tile - 1) & 1, ctl);
+          ok = ok && wait_phase(&empty[st], ((ph >> st) & 1) ^ 1, ctl);
+          if (!ok) break;
+          mbar_expect_tx(&full[st], A_BYTES + x.halves * B_BYTES);
+          uint8_t* sa = tiles + (size_t)st * STAGE_BYTES;
+          // all four digit tiles of an operand in one copy
+          const int kc = (x.kb0 + kb) * KSTAGE;
+          tma_load_4d(&tma_a, &full[st], sa, kc, x.m0, x.ub);
+          tma_load_4d(&tma_b, &full[st], sa + A_BYTES, kc, x.n0, x.vb);
+          if (x.halves == 2) tma_load_4d(&tma_b, &full[st], sa + A_BYTES + B_BYTES, kc, x.n0 + HN, x.vb);
+          ph ^= 1u << st;
+          live |= 1u << st;
+          st = st + 1 == STAGES ? 0 : st + 1;
+        }
       }
       if (ctl->abort) {
         // let the copies this thread issued land before the CTA exits
-        for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-          wait_phase(&full[kb % STAGES], (kb / STAGES) & 1, ctl, kTimeoutCycles / 2);
+        for (int s = 0; s < STAGES; ++s)
+          if ((live >> s) & 1) wait_phase(&full[s], ((ph >> s) & 1) ^ 1, ctl, kTimeoutCycles / 2);
       }
     }
-  } else if (warp <= halves) {
+  } else if (warp <= H) {
     // ------------------------------------------------------------ MMA issuers
     // warp 1 + h issues half h: a thread that waits for one half's drain leaves
     // the other's MMAs flowing
@@ -239,34 +290,49 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
       const int h = warp - 1;
       const uint32_t ab = su32(tiles);
       const uint32_t acc = tmem + 4 * HN * h;
-      // the epilogue warps have zeroed the accumulators
-      bool ok = wait_phase(zero_done, 0, ctl);
-      for (int kb = 0; ok && kb < n_kb; ++kb) {
-        const int st = kb % STAGES;
-        ok = wait_phase(&full[st], (kb / STAGES) & 1, ctl);
-        if (!ok) break;
-        tc_fence_after();
-        const uint64_t da = sdesc64(ab + st * STAGE_BYTES);
-        const uint64_t db = sdesc64(ab + st * STAGE_BYTES + A_BYTES + h * B_BYTES);
-        // the digits that touch only diagonals 2 and 3 do not wait for the
-        // half's drain (but the second does for a fold)
-        const bool folding = kb % kFold == 0;
-        mma_digit<3>(acc, da, db);
-        if (!folding) mma_digit<2>(acc, da, db);
-        if (kb > 0) {
-          ok = wait_phase(&drained[h], (kb - 1) & 1, ctl);
-          if (!ok) break;
-          tc_fence_after();
+      uint32_t ph = 0, it = 0;  // bit s of ph: parity of stage s's next use
+      bool ok = true;
+      for (uint32_t t = blockIdx.x; ok && t < args.tiles; t += gridDim.x, ++it) {
+        int n_kb;
+        bool mine;
+        {
+          const Tile x = tile_at(t);
+          n_kb = x.n_kb, mine = h < x.halves;
         }
-        if (folding) mma_digit<2>(acc, da, db);
-        mma_digit<1>(acc, da, db);
-        mma_digit<0>(acc, da, db);
-        if (kb + 1 < n_kb) tc_commit(&go[h]);
-        tc_commit(&empty[st]);
+        // the epilogue warps have read out the last tile and zeroed the accumulators
+        ok = wait_phase(zero_done, it & 1, ctl);
+        int st = C::FIRST;
+        for (int kb = 0; ok && kb < n_kb; ++kb) {
+          ok = wait_phase(&full[st], (ph >> st) & 1, ctl);
+          if (!ok) break;
+          ph ^= 1u << st;
+          tc_fence_after();
+          if (mine) {
+            const uint64_t da = sdesc64(ab + st * STAGE_BYTES);
+            const uint64_t db = sdesc64(ab + st * STAGE_BYTES + A_BYTES + h * B_BYTES);
+            // the digits that touch only diagonals 2 and 3 do not wait for the
+            // half's drain (but the second does for a fold)
+            const bool folding = kb > 0 && !(kb & 1) && folds_after(n_kb - 1 - kb);
+            mma_digit<3>(acc, da, db);
+            if (!folding) mma_digit<2>(acc, da, db);
+            if (kb > 0) {
+              ok = wait_phase(&drained[h], (kb - 1) & 1, ctl);
+              if (!ok) break;
+              tc_fence_after();
+            }
+            if (folding) mma_digit<2>(acc, da, db);
+            mma_digit<1>(acc, da, db);
+            mma_digit<0>(acc, da, db);
+            // (an even number of phases a tile: the drains' parities start from 0)
+            if (kb + 1 < n_kb || (kb & 1)) tc_commit(&go[h]);
+          }
+          tc_commit(&empty[st]);
+          st = st + 1 == STAGES ? 0 : st + 1;
+        }
+        tc_commit(acc_full);
+        // (keeps the MMAs in flight from outliving the CTA after an abort)
+        if (!ok) wait_phase(acc_full, it & 1, ctl, kTimeoutCycles / 2);
       }
-      tc_commit(acc_full);
-      // (also keeps the MMAs in flight from outliving the CTA after an abort)
-      wait_phase(acc_full, 0, ctl, kTimeoutCycles / 2);
     }
   } else if (warp >= EPI_WARP0) {
     // ------------------------------------------------------------ epilogue
@@ -283,8 +349,6 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
     // K they gain 2^15 and 2^16 + 3 x 2^5 at most, and every fold carries s1
     // into s0: int32 holds a K range of up to 32768 columns.
     int32_t s0[32], s1[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) s0[j] = s1[j] = 0;
     const float M8 = 100663296.0f;             // 1.5 * 2^26: ulp 8, |x| <= 2^25
     const int32_t B8 = (int32_t)__float_as_uint(M8);
     const float M0 = 12582912.0f;              // 1.5 * 2^23: ulp 1
@@ -302,9 +366,9 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
     // The half after stage kb: its diagonal 1 (32 columns of this thread) and
     // every second stage, in turns, 16 of diagonal 0; all of diagonal 2 after
     // kFold stages.
-    auto drain = [&](auto ODD, int kb) {
+    auto drain = [&](auto ODD, int left) {
       constexpr int o = decltype(ODD)::value * 16;
-      if (!wait_phase_sleep(&go[h], (uint32_t)kb & 1, ctl)) return false;
+      if (!wait_phase_sleep(&go[h], decltype(ODD)::value, ctl)) return false;
       tc_fence_after();
       uint32_t a[16];
       auto drain_at = [&](uint32_t at, int32_t* s) {
@@ -317,7 +381,7 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
       drain_at(lane_base + HN, s1);
       drain_at(lane_base + HN + 16, s1 + 16);
       drain_at(lane_base + o, s0 + o);
-      if (o != 0 && (kb + 1) % kFold == 0) {
+      if (o != 0 && folds_after(left)) {
         // diagonal 2 (the MMAs that write it wait): multiples of 2^13 = 8 x 2^10
         // to s1, |rest| <= 2^12 stays
 #pragma unroll
@@ -345,9 +409,8 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
       return true;
     };
     static_assert(kFold % 2 == 0, "folds follow odd stages");
-    bool ok = true;
-    if (h < halves) {
-      // the accumulators start from zero (every MMA accumulates)
+    // the accumulators start from zero (every MMA accumulates)
+    auto zero = [&] {
 #pragma unroll
       for (int d = 0; d < 4; ++d)
 #pragma unroll
@@ -356,96 +419,154 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(zero_done);
+    };
+    zero();
+    bool ok = true;
+    // stages of tile t for the half of epilogue thread et
+    auto my_stages = [&](uint32_t t, int et) {
+      const Tile x = tile_at(t);
+      return (et >> 8) < x.halves ? x.n_kb : 0;
+    };
+    for (uint32_t it = 0;; ++it) {
+      int left;          // drains to come
+      {
+        const uint32_t t = blockIdx.x + it * gridDim.x;
+        if (t >= args.tiles) break;
+        const Tile x = tile_at(t);
+        const int et = tid_again() - EPI_WARP0 * 32;
+        left = my_stages(t, et) - 1;
+        // this tile's offsets in W and exponents, beside the last one's, which other
+        // warps may still read
+        int64_t* coff = (int64_t*)(tabs + (it & 1) * C::TAB);
+        int64_t* roffs = coff + TN;
+        int32_t* cexp = (int32_t*)(roffs + TM);
+        int32_t* rexps = cexp + TN;
+        if (et < TM) {
+          const bool rok = x.m0 + et < p.M;
+          roffs[et] = rok ? args.wrow[(int64_t)x.b * p.M + x.m0 + et] : -1;
+          rexps[et] = rok ? args.eu[(int64_t)x.ub * p.M + x.m0 + et] - kExpBias : 0;
+          if (et < TN) {
+            const bool cok = x.n0 + et < p.N;
+            coff[et] = cok ? args.wcol[(int64_t)x.b * p.N + x.n0 + et] : -1;
+            cexp[et] = cok ? args.ev[(int64_t)x.vb * p.N + x.n0 + et] - kExpBias : 0;
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 32; ++j) s0[j] = s1[j] = 0;
       // two stages a turn: the parts of diagonal 0 are compile-time
-      for (int kb = 0; ok && kb + 1 < n_kb; kb += 2) {
-        ok = drain(std::integral_constant<int, 0>{}, kb);
-        if (ok && kb + 2 < n_kb) ok = drain(std::integral_constant<int, 1>{}, kb + 1);
-      }
-    }
-    if (ok) ok = wait_phase_sleep(acc_full, 0, ctl);
-    ok = ok && !ctl->abort;
-    if (ok && h < halves) {
-      tc_fence_after();
-      // The last stages and the running sums as one int64 in units of 2^-20,
-      // staged through shared memory (the operand stages are free by now).
-      int64_t* st64 = (int64_t*)tiles + row * LD + h * HN + part * 32;
-#pragma unroll
-      for (int pc = 0; pc < 8; ++pc) {
-        uint32_t a0[4], a1[4], a2[4], a3[4];
-        const uint32_t at = lane_base + pc * 4;
-        tmem_ld4(at, a0);
-        tmem_ld4(at + HN, a1);
-        tmem_ld4(at + 2 * HN, a2);
-        tmem_ld4(at + 3 * HN, a3);
-        tmem_wait_ld();
-        tmem_loaded<4>(a0);
-        tmem_loaded<4>(a1);
-        tmem_loaded<4>(a2);
-        tmem_loaded<4>(a3);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          // multiples of 8 of the exact diagonals by the magic number, as in the
-          // drains, their rests (an integer below 2^13) likewise; diagonals 2 and 3
-          // (|.| < 2^29) as one FP32 number and the only conversion
-          const float x0 = __uint_as_float(a0[j]), x1 = __uint_as_float(a1[j]);
-          const float r0 = x0 + M8, r1 = x1 + M8;
-          const int32_t t0 = s0[pc * 4 + j] + ((int32_t)__float_as_uint(r0) - B8);
-          const int32_t t1 = s1[pc * 4 + j] + ((int32_t)__float_as_uint(r1) - B8);
-          const float low = __fmaf_rn(__uint_as_float(a3[j]), 1.0f / 1024.0f, __uint_as_float(a2[j]));
-          const float rest = __fmaf_rn(x0 - (r0 - M8), 1024.0f, x1 - (r1 - M8));
-          const int32_t l = (((int32_t)__float_as_uint(rest + M0) - B0) << 10) + __float2int_rn(low);
-          st64[pc * 4 + j] = ((long long)t0 << 23) + ((long long)t1 << 13) + l;
-        }
-      }
-    }
-    tc_fence_before();
-    // all epilogue threads meet here, whatever path they took
-    asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
-    if (ok) {
-      // a warp per row: lane l rounds and writes columns l, l + 32, ...; two rows
-      // at a time (one was bound by the latency of its conversions)
-      constexpr int NC = TN / 32;
-      const int nrow = (int)min((int64_t)TM, p.M - m0), ncol = (int)min((int64_t)TN, p.N - n0);
-      const long long* R0 = (const long long*)tiles + lane;
-      if (args.ksplit > 1) {
-        unsigned long long* acc = args.wacc + ((int64_t)zb * p.M + m0) * p.N + n0 + lane;
 #pragma unroll 1
-        for (int r = ew; r < nrow; r += EPI_WARPS) {
+      while (ok && left > 0) {
+        ok = drain(std::integral_constant<int, 0>{}, --left);
+        if (ok && left > 0) ok = drain(std::integral_constant<int, 1>{}, --left);
+      }
+      // the thread's place and its tile again: they would not fit the registers
+      // beside the sums
+      const int et = tid_again() - EPI_WARP0 * 32;
+      const uint32_t t = blockIdx.x + it * gridDim.x;
+      const int n_kb = my_stages(t, et);
+      const bool extra = n_kb != 0 && !(n_kb & 1);   // the phase that makes them even
+      if (ok && extra) ok = wait_phase_sleep(&go[h], 1, ctl);
+      if (ok) ok = wait_phase_sleep(acc_full, it & 1, ctl);
+      ok = ok && !ctl->abort;
+      tc_fence_after();
+      const int ew = et >> 5, lane = et & 31;
+      if (ok && n_kb != 0) {
+        // The last stages and the running sums as one int64 in units of 2^-20,
+        // staged through shared memory (the operand stages are free by now): row r's
+        // column c at word c ^ (r % 32), so that both walks spread over the banks.
+        const int row = et & (TM - 1), part = (et >> 7) & 1;
+        int64_t* st64 = (int64_t*)tiles + row * TN + (et >> 8) * HN + part * 32;
 #pragma unroll
-          for (int j = 0; j < NC; ++j)
-            if (lane + 32 * j < ncol)
-              red_add_u64(acc + (int64_t)r * p.N + 32 * j, (unsigned long long)R0[r * LD + 32 * j]);
+        for (int pc = 0; pc < 8; ++pc) {
+          uint32_t a0[4], a1[4], a2[4], a3[4];
+          const uint32_t at = lane_base + pc * 4;
+          tmem_ld4(at, a0);
+          tmem_ld4(at + HN, a1);
+          tmem_ld4(at + 2 * HN, a2);
+          tmem_ld4(at + 3 * HN, a3);
+          tmem_wait_ld();
+          tmem_loaded<4>(a0);
+          tmem_loaded<4>(a1);
+          tmem_loaded<4>(a2);
+          tmem_loaded<4>(a3);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            // multiples of 8 of the exact diagonals by the magic number, as in the
+            // drains, their rests (an integer below 2^13) likewise; diagonals 2 and 3
+            // (|.| < 2^29) as one FP32 number and the only conversion
+            const float x0 = __uint_as_float(a0[j]), x1 = __uint_as_float(a1[j]);
+            const float r0 = x0 + M8, r1 = x1 + M8;
+            const int32_t t0 = s0[pc * 4 + j] + ((int32_t)__float_as_uint(r0) - B8);
+            const int32_t t1 = s1[pc * 4 + j] + ((int32_t)__float_as_uint(r1) - B8);
+            const float low = __fmaf_rn(__uint_as_float(a3[j]), 1.0f / 1024.0f, __uint_as_float(a2[j]));
+            const float rest = __fmaf_rn(x0 - (r0 - M8), 1024.0f, x1 - (r1 - M8));
+            const int32_t l = (((int32_t)__float_as_uint(rest + M0) - B0) << 10) + __float2int_rn(low);
+            st64[(pc * 4 + j) ^ lane] = ((long long)t0 << 23) + ((long long)t1 << 13) + l;
+          }
         }
-      } else {
-        OutMode wp;
-        wp.negate = args.neg[part_v];
-        wp.accumulate = p.accumulate;
-        int64_t co[NC];
-        int ce[NC];
+      }
+      // the next tile's MMAs may start
+      if (t + gridDim.x < args.tiles) {
+        if (lane == 0 && extra) mbar_arrive(&drained[h]);
+        zero();
+      }
+      ok = all_ok<EPI_WARPS * 32>(ok);
+      if (ok) {
+        const Tile x = tile_at(t);
+        const int64_t* coff = (const int64_t*)(tabs + (it & 1) * C::TAB);
+        const int64_t* roffs = coff + TN;
+        const int32_t* cexp = (const int32_t*)(roffs + TM);
+        const int32_t* rexps = cexp + TN;
+        // a warp per row: lane l rounds and writes columns l, l + 32, ...; two rows
+        // at a time (one was bound by the latency of its conversions)
+        constexpr int NC = TN / 32;
+        const int nrow = (int)min((int64_t)TM, p.M - x.m0), ncol = (int)min((int64_t)TN, p.N - x.n0);
+        const long long* R0 = (const long long*)tiles;
+        if (args.ksplit > 1) {
+          unsigned long long* acc = args.wacc + ((int64_t)x.vb * p.M + x.m0) * p.N + x.n0 + lane;
+#pragma unroll 1
+          for (int r = ew; r < nrow; r += EPI_WARPS) {
 #pragma unroll
-        for (int j = 0; j < NC; ++j) co[j] = coff[lane + 32 * j], ce[j] = cexp[lane + 32 * j] - 36;
+            for (int j = 0; j < NC; ++j)
+              if (lane + 32 * j < ncol)
+                red_add_u64(acc + (int64_t)r * p.N + 32 * j, (unsigned long long)R0[r * TN + 32 * j + (lane ^ (r & 31))]);
+          }
+        } else {
+          OutMode wp;
+          wp.negate = args.neg[x.part];
+          wp.accumulate = p.accumulate;
+          int64_t co[NC];
+          int ce[NC];
+#pragma unroll
+          for (int j = 0; j < NC; ++j) co[j] = coff[lane + 32 * j], ce[j] = cexp[lane + 32 * j] - 36;
 #pragma unroll 2
-        for (int r = ew; r < nrow; r += EPI_WARPS) {
-          const int64_t ro = roffs[r];
-          const int re = rexps[r];
-          long long R[NC];
-          int ex[NC];
-          double d[NC];
+          for (int r = ew; r < nrow; r += EPI_WARPS) {
+            const int64_t ro = roffs[r];
+            const int re = rexps[r];
+            long long R[NC];
+            int ex[NC];
+            double d[NC];
 #pragma unroll
-          for (int j = 0; j < NC; ++j) R[j] = R0[r * LD + 32 * j], ex[j] = re + ce[j];
-          i64_scaled_batch<NC>(R, ex, d);
-          if (ro < 0) continue;   // general plans: a row absent from W
+            for (int j = 0; j < NC; ++j) R[j] = R0[r * TN + 32 * j + (lane ^ (r & 31))], ex[j] = re + ce[j];
+            i64_scaled_batch<NC>(R, ex, d);
+            if (ro < 0) continue;   // general plans: a row absent from W
 #pragma unroll
-          for (int j = 0; j < NC; ++j) {
-            if (co[j] < 0) continue;   // beyond N, or a column absent from W
-            if constexpr (!GEN) {
-              args.w[ro + co[j]] = d[j];
-            } else {
-              store_w(wp, args.w + args.woff[part_v] + (int64_t)p.es * (ro + co[j]), d[j]);
+            for (int j = 0; j < NC; ++j) {
+              if (co[j] < 0) continue;   // beyond N, or a column absent from W
+              if constexpr (!GEN) {
+                args.w[ro + co[j]] = d[j];
+              } else {
+                store_w(wp, args.w + args.woff[x.part] + (int64_t)p.es * (ro + co[j]), d[j]);
+              }
             }
           }
         }
       }
+      if (!ok || t + gridDim.x >= args.tiles) break;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // TMA writes there next
+      __syncwarp();
+      if (lane == 0) mbar_arrive(staged);
     }
   }
   // a split-K rounding kernel behind this one may start its launch now
@@ -499,9 +620,14 @@ cudaError_t launch_mode(const Problem& p, const Tables& tab, const void* a, cons
   }
   const int64_t gx = (p.N + TN - 1) / TN, gy = (p.M + TM - 1) / TM;
   const int64_t gz = (int64_t)args.parts * p.n_q * args.ksplit;
-  if (gx > 0x7FFFFFFF || gy > 65535 || gz > 65535) return cudaErrorInvalidConfiguration;
+  if (gx > 0x7FFFFFFF || gy > 65535 || gz > 65535 || gx * gy > 0x7FFFFFFFll / gz) return cudaErrorInvalidConfiguration;
+  args.gx = (int)gx;
+  args.gy = (int)gy;
+  args.tiles = (uint32_t)(gx * gy * gz);
+  // persistent CTAs, each walking the tiles one grid apart
+  const int64_t resident = (int64_t)device_sms() * (3 - H);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)gx, (unsigned)gy, (unsigned)gz);
+  cfg.gridDim = dim3((unsigned)(args.tiles < resident ? args.tiles : resident));
   cfg.blockDim = dim3(C::NTHREADS);
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = st;

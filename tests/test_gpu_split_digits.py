@@ -83,3 +83,24 @@ def test_narrow_tiles(sc, M, N, K):
     for q in range(G):
         bound = K * 2.0 ** -36 * 64.0    # |entries| < 8 = 2^(E+1)
         assert np.all(np.abs(w[q] - u[q] @ v[q]) <= bound)
+
+
+@pytest.mark.parametrize("K", [20, 64, 90, 545, 1056])
+@pytest.mark.parametrize("M,N", [(1300, 1172), (19300, 40)])
+def test_several_tiles_per_cta(sc, M, N, K):
+    """Three irreps in more tiles than stay resident, so that a CTA walks several:
+    full ones and ones with half their columns or a few rows, of 1, 2, 3, 18 and 33
+    stages (K ranges of odd and even length start the next tile's waits); the second
+    shape takes the narrow kernel.  The same bound as above."""
+    G = 3
+    p = sc.Plan("ij,jk->ik", (G,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
+    rng = np.random.default_rng(K)
+    u, v = rng.standard_normal(p.shape_u), rng.standard_normal(p.shape_v)
+    ud, vd = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+    w = p.contract(ud, vd)
+    again = p.contract(ud, vd)
+    p.check_device_error()
+    assert torch.equal(w, again)
+    w = w.cpu().numpy()
+    for q in range(G):
+        assert np.all(np.abs(w[q] - u[q] @ v[q]) <= K * 2.0 ** -36 * 64.0)
