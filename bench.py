@@ -201,6 +201,7 @@ KERNEL_SOURCES = {
     "rowstream_kernel": ("transforms.cu", "symctr_internal.h"),
     "gemm_tc_kernel": ("gemm_tc.cu", "tc_common.cuh", "symctr_internal.h"),
     "gemm_tc10_kernel": ("gemm_tc10.cu", "tc_common.cuh", "symctr_internal.h"),
+    "gemm_tf32_direct_kernel": ("gemm_tf32_direct.cu", "transforms.cu", "tc_common.cuh", "symctr_internal.h"),
     "gemm_f64": ("gemm_f64.cu", "symctr_internal.h"),
 }
 
@@ -258,7 +259,25 @@ def prep_bytes(pl):
     elems = i.aligned_numel_u + i.aligned_numel_v
     if i.precision == 1:
         return elems * (8 + 2 * digit_planes(i.n_slices)) + 4 * i.n_q * (i.M + i.N)
+    direct = tf32_direct(pl)
+    if direct is not None:
+        elems = (i.aligned_numel_v, i.aligned_numel_u)[direct]
     return elems * (8 + 4)
+
+
+def tf32_direct(pl):
+    """The operand (0 or 1) whose float64 entries the TF32 GEMM reads itself, or
+    None: the shape rule of tf32_direct_operand in transforms.cu (one pass, real,
+    uniform plans)."""
+    i = pl.info
+    inputs = pl.einsum.replace(" ", "").split("->")[0].split(",")
+    for op in (0, 1):
+        rows, other = ((i.M, i.N), (i.N, i.M))[op]
+        last, dim = inputs[op][-1], (pl.sym_u, pl.sym_v)[op].dims[-1]
+        if other <= 512 and rows >= 4 * other and (rows + 127) // 128 * i.n_q >= 128 and i.K >= 64 \
+                and last in inputs[1 - op] and dim % 2 == 0:
+            return op
+    return None
 
 
 def prep_kernels(pl):
@@ -297,7 +316,8 @@ def rooflines(args, plans, prep, gemm, pk):
         peak_src = f"{pk['src']} bf16 burst"
     elif args.precision == "tf32":
         work = sum(pl.useful_flops for pl in plans)
-        kernel, bound, unit, peak = "gemm_tc_kernel", "tensor", "TFLOP/s", pk["bf16_tflops"] / 2
+        kernel = "gemm_tc_kernel" if tf32_direct(plans[0]) is None else "gemm_tf32_direct_kernel"
+        bound, unit, peak = "tensor", "TFLOP/s", pk["bf16_tflops"] / 2
         peak_src = f"{pk['src']} bf16 burst x 1/2 (nominal tf32:bf16 ratio)"
     else:
         work = sum(pl.useful_flops for pl in plans)

@@ -427,7 +427,7 @@ int64_t gcd64(int64_t a, int64_t b) {
 // the front, irrep by irrep, and M, N and K shrink to the largest count; -1
 // fills the other irreps up.  (Absent entries of W are zeros that the zero fill
 // writes.)  The ladder with 8 x 24 virtual, 8 x 8 occupied indices, sub-group
-// modes and ragged sectors: 4608 x 512 x 4608 -> 1285 x 192 x 738 per irrep, 2.32 -> 0.13 ms.
+// modes and ragged sectors: 4608 x 512 x 4608 -> 1285 x 192 x 738 per irrep, 2.32 -> 0.10 ms.
 void compact_tables(symctr_plan* P, std::vector<int64_t>& whole) {
   const Problem& pr = P->prob;
   P->run = pr;
