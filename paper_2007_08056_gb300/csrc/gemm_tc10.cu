@@ -42,8 +42,8 @@
 // the tensor pipe empty, 2970 for the five BF16 digits before.  Float-to-int
 // conversions run at 16 per clock and SM here, so the drains use magic-number
 // adds (3470 with conversions).  CC ladder step 6.68 -> 5.49 ms, (2,2,2) with
-// D = 23 1.02 -> 0.81 ms, 40960 x 640 x 640 by 10 irreps 5.11 -> 3.70 ms (3.99
-// with a CTA to a tile, whose setup, first loads and writes nothing covered).
+// D = 23 1.02 -> 0.81 ms, 40960 x 640 x 640 by 10 irreps 5.11 -> 3.59 ms (3.99
+// with a CTA to a tile and the longer writes, 3.70 with those alone).
 // The drain loop leaves no register to spare: with 80 bytes of spills instead of
 // 32 that last case takes 4.01 ms.
 // Every wait is bounded (see tc_common.cuh).
@@ -144,6 +144,36 @@ struct Tc10Args {
   int gx, gy;        // column and row blocks
   uint32_t tiles;    // gx * gy * parts * n_q * ksplit
 };
+
+// Rv[j] * 2^e[j] as float64 (exact) for |Rv| < 2^53 and results that are 0 or
+// normal; false if an even entry is not in [-2^51, 2^51).  The selects and shifts of the integer way run at half rate and took
+// most of a tile's write phase (11300 clocks); every second value goes through
+// the float64 pipe instead, which is otherwise idle (one addition against
+// 1.5 * 2^52, 2 per clock and SM, so not all of them: 16384 would take 8200).
+// 40960 x 640 x 640 by 10 irreps 3.70 -> 3.59 ms (3.79 with all of them there),
+// the CC ladder with 16 irreps and gradients 6.08 -> 5.90 ms.
+template <int B>
+__device__ __forceinline__ bool i64_scaled_small(const long long (&Rv)[B], const int (&e)[B], double (&d)[B]) {
+  uint32_t out = 0;
+#pragma unroll
+  for (int j = 0; j < B; ++j) {
+    const uint32_t lo = (uint32_t)Rv[j], hi = (uint32_t)((unsigned long long)Rv[j] >> 32);
+    if (j % 2 == 0) {
+      out |= (hi + 0x43380000u) ^ 0x43300000u;
+      const double x = __hiloint2double((int)(hi + 0x43380000u), (int)lo) - 6755399441055744.0;
+      const int h = __double2hiint(x);
+      d[j] = __hiloint2double(h == 0 ? 0 : h + (e[j] << 20), __double2loint(x));
+    } else {
+      const uint64_t sm = (uint64_t)(Rv[j] >> 63);
+      const uint64_t m = ((uint64_t)Rv[j] ^ sm) - sm;
+      const int lz = __clzll((long long)m);
+      const uint64_t q = m << ((lz - 11) & 63);     // the leading one at bit 52
+      const uint32_t h = (uint32_t)(q >> 32) + ((uint32_t)(e[j] + 63 - lz + 1022) << 20);
+      d[j] = __hiloint2double((int)(m == 0 ? 0u : h | ((uint32_t)sm & 0x80000000u)), (int)(uint32_t)q);
+    }
+  }
+  return out >> 20 == 0;
+}
 
 // The thread's index, read again.
 __device__ __forceinline__ int tid_again() {
@@ -538,8 +568,14 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
           wp.accumulate = p.accumulate;
           int64_t co[NC];
           int ce[NC];
+          int clo = INT32_MAX / 2, chi = INT32_MIN / 2;   // of the columns that are not all zero
 #pragma unroll
-          for (int j = 0; j < NC; ++j) co[j] = coff[lane + 32 * j], ce[j] = cexp[lane + 32 * j] - 36;
+          for (int j = 0; j < NC; ++j) {
+            co[j] = coff[lane + 32 * j], ce[j] = cexp[lane + 32 * j] - 36;
+            if (ce[j] > -kExpBias - 36) clo = min(clo, ce[j]), chi = max(chi, ce[j]);
+          }
+          // |R| <= 2^38 per column of K, and less than one more for what was dropped
+          const bool small = args.kb_per_split * KSTAGE < 32768;
 #pragma unroll 2
           for (int r = ew; r < nrow; r += EPI_WARPS) {
             const int64_t ro = roffs[r];
@@ -549,7 +585,9 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
             double d[NC];
 #pragma unroll
             for (int j = 0; j < NC; ++j) R[j] = R0[r * TN + 32 * j + (lane ^ (r & 31))], ex[j] = re + ce[j];
-            i64_scaled_batch<NC>(R, ex, d);
+            // (an all-zero row's R are 0 whatever its exponent)
+            const bool normal = re <= -kExpBias || (re + clo >= -1022 && re + chi <= 969);
+            if (!(small && normal && i64_scaled_small<NC>(R, ex, d))) i64_scaled_batch<NC>(R, ex, d);
             if (ro < 0) continue;   // general plans: a row absent from W
 #pragma unroll
             for (int j = 0; j < NC; ++j) {

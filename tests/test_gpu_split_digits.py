@@ -104,3 +104,21 @@ def test_several_tiles_per_cta(sc, M, N, K):
     w = w.cpu().numpy()
     for q in range(G):
         assert np.all(np.abs(w[q] - u[q] @ v[q]) <= K * 2.0 ** -36 * 64.0)
+
+
+@pytest.mark.parametrize("N", [70, 40])
+def test_row_and_column_scales_to_the_ends_of_the_range(sc, N):
+    """Small integers times powers of two, with zero rows and columns: the sums are
+    exact, so every result is the sum rounded once, normal, subnormal or 0."""
+    M, K = 130, 64
+    rng = np.random.default_rng(N)
+    u, v = (rng.integers(-31, 32, (r, K)).astype(np.float64) for r in (M, N))
+    a = np.resize([-600, -511, -480, 0, 490, 505, -540], M)
+    b = np.resize([0, -560, -511, -470, 480, 495], N)
+    u[5], u[64], v[3], v[N - 1] = 0, 0, 0, 0
+    p = sc.Plan("ij,jk->ik", (1,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
+    us, vs = np.ldexp(u, a[:, None]), np.ldexp(v, b[:, None])
+    w = p.contract(torch.from_numpy(us).cuda().reshape(p.shape_u),
+                   torch.from_numpy(np.ascontiguousarray(vs.T)).cuda().reshape(p.shape_v))
+    p.check_device_error()
+    assert np.array_equal(w.cpu().numpy().reshape(M, N), np.ldexp(u @ v.T, a[:, None] + b[None, :]))
