@@ -1,7 +1,7 @@
 """The TF32 form that reads its long operand's float64 entries itself: both
-roles, one and two MMAs per tile, ragged row tiles, K not a multiple of a stage or an offset chunk, zeros, entries
-beyond FP32's normal range, and the shapes next to its rule, which take the
-two-step path.  Products of TF32-rounded operands (relative 2^-11 each) summed in
+roles, one and two MMAs per tile, ragged row tiles, K not a multiple of a stage
+or an offset chunk, zeros, entries beyond FP32's normal range, and the shapes
+next to its rule, which take the two-step path.  Products of TF32-rounded operands (relative 2^-11 each) summed in
 FP32: within K-independent 2^-10 of |u| |v|, plus 2^-20 K^(1/2) of it for the
 sums."""
 import numpy as np
