@@ -6,22 +6,29 @@
 // Why FP16 and base 1024.  The operand keeps 39 bits and a sign whatever the
 // digits are.  BF16 holds 8 significant bits, so it needs 5 digits and 15
 // slice pairs (i + j <= 4); FP16 holds 11, and four balanced digits a_i in
-// [-512, 512] need 10 pairs (i + j <= 3): two thirds of the tensor work, and
+// [-512, 511] need 10 pairs (i + j <= 3): two thirds of the tensor work, and
 // four planes instead of five to write and read.  What bounds the digit is the
 // FP32 accumulator: it adds integers exactly up to 2^24, i.e. 64 products of
-// 2^18.  The dropped pairs (i + j = 4, three of them) weigh 3 x 2^-40 of the
-// largest product, against 4 x 2^-40 (four pairs) with 8-bit digits.
+// just below 2^18.  The dropped pairs (i + j = 4, three of them) weigh 3 x 2^-40
+// of the largest product, against 4 x 2^-40 (four pairs) with 8-bit digits.
 //
-// Diagonals d = i + j, each in its own TMEM accumulator:
-//   d = 0  one pair, <= 2^18 per K: drained every 64 columns of K
-//   d = 1  two pairs, <= 2^19 per K: drained every 32 columns (every stage)
-//   d = 2  three pairs (weight 2^-20): its multiples of 2^13 move into the sum
-//          of diagonal 1 every kFold stages (exact), the rest stays
+// Diagonals d = i + j, each in its own TMEM accumulator; the leading digit is at
+// most 511 (row_exponent raises a row's scale where it would be 512):
+//   d = 0  one pair, <= 511^2 per K: drained every 64 columns of K,
+//          64 x 511^2 + 4 = 2^24 - 65468
+//   d = 1  two pairs, <= 2 x 511 x 512 per K: drained every 32 columns (every
+//          stage), 32 x 2 x 511 x 512 + 4 = 2^24 - 32764
+//   d = 2  three pairs (weight 2^-20): an FP32 sum that reaches 3 x 2^27 in 17
+//          stages and is then rounded to 2^5 in each MMA, 2^-37 of its 16
+//          largest products at worst (lower digits all at their limits and of
+//          one sign; random ones stay below 2^24 and exact); its multiples of
+//          2^13 move into the sum of diagonal 1 every kFold stages, the rest stays
 //   d = 3  four pairs (weight 2^-30): rounded at 2^-24 of its sum, 2^-54 in all
 // A drain moves the accumulator's multiple of 8 into an int32 and leaves the
-// rest, so the sums are exact.  At the end they make one int64 in units of
-// 2^-20 of the d = 0 unit, rounded once to float64 with the row and column
-// exponents (integer arithmetic only: GB300 has little float64 throughput).
+// rest of at most 4, so the sums of diagonals 0 and 1 are exact.  At the end all
+// make one int64 in units of 2^-20 of the d = 0 unit, rounded once to float64
+// with the row and column exponents (integer arithmetic only: GB300 has little
+// float64 throughput).
 //
 // CTA: 640 threads: warp 0 TMA, warps 1 and 2 MMA, warps 4-19 drains and
 // epilogue; 128 x 128 tiles, 512 TMEM columns, three stages of 64 KB.  The grid is

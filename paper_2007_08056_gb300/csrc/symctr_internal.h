@@ -269,6 +269,32 @@ constexpr int kMaxSlices = 6;
 // and a sign) holds four FP16 digits of 10 bits, the others n_slices BF16
 // digits of 8 bits.
 inline int digit_planes(int n_slices) { return n_slices == 5 ? 4 : n_slices; }
+
+// Binary exponent E of an aligned row (every |x| < 2^(E+1)) from the bit pattern
+// `ab` of its largest finite |x| > 0, whose low word counts only when the high
+// one is zero.  E is clamped below at 8S - 1076: a row whose largest entry is
+// smaller holds only subnormals, which are exact integers at that scale
+// (multiples of 2^-1074), so nothing is lost.
+// Default split: E is one more where the largest entry, rounded to 39 bits,
+// might have the leading digit 512, i.e. from 1 - 2^-10 - 2^-20 - 2^-30 of
+// 2^(E+1) on (the high word's unit allowed for).  Leading digits up to 511 are
+// what the accumulators of diagonals 0 and 1 have room for (gemm_tc10.cu):
+// entries near a power of two from below, all of one sign, would overflow them.
+SC_HD int row_exponent(uint64_t ab, int S) {
+  const int ef = (int)(ab >> 52);
+  const uint64_t m = ef != 0 ? (ab & ((1ull << 52) - 1)) | (1ull << 52) : ab;
+#if defined(__CUDA_ARCH__)
+  const int nb = 64 - __clzll((long long)m);
+#else
+  const int nb = 64 - __builtin_clzll(m);
+#endif
+  int e = ef != 0 ? ef - 1023 : nb - 1 - 1074;
+  if (S == 5) {
+    const uint64_t most = m | 0xFFFFFFFFull;     // the largest entry with this high word
+    if (nb > 32 && ((most << (64 - nb)) >> 43) >= 0x1FF7FDull) ++e;
+  }
+  return e > 8 * S - 1076 ? e : 8 * S - 1076;
+}
 constexpr int kKBlock = 32;         // K per pipeline stage (64-byte rows of BF16)
 constexpr int kKChunk = 64;         // K between exact flushes of the top accumulators
 

@@ -116,8 +116,7 @@ __global__ void __launch_bounds__(THREADS) align_kernel(Problem p, OperandMap m,
 // ---------------------------------------------------------------------------
 
 // Row exponents, stored biased: E + kExpBias for a row whose largest entry
-// lies in [2^E, 2^(E+1)) (E clamped below at 8S - 1076, see row_key), 0 for an
-// all-zero row.
+// lies below 2^(E+1) (see row_exponent), 0 for an all-zero row.
 constexpr int32_t kExpBias = 4096;
 constexpr int SCAN_COLS = 256;
 constexpr int SLICE_COLS = 64;
@@ -148,10 +147,8 @@ struct Max2 {
 };
 
 // Biased row exponent key from the largest |x| bit pattern of a row: 0 for an
-// all-zero row; nonfinite entries set `bad`.  E is clamped below at 8S - 1076:
-// a row whose largest entry is smaller holds only subnormals, which are exact
-// integers at that scale (multiples of 2^-1074), so nothing is lost, and every
-// entry then needs a right shift only (fixed_point).
+// all-zero row; nonfinite entries set `bad`.  The exponent's lower clamp
+// (row_exponent) leaves every entry a right shift only (fixed_point).
 template <int S>
 __device__ __forceinline__ int32_t row_key(uint64_t ab, unsigned& bad) {
   if (ab == 0) return 0;
@@ -159,9 +156,7 @@ __device__ __forceinline__ int32_t row_key(uint64_t ab, unsigned& bad) {
     bad = 1;
     return 0;
   }
-  const int ef = (int)(ab >> 52);
-  const int e = ef != 0 ? ef - 1023 : (63 - __clzll((long long)ab)) - 1074;
-  return max(e, 8 * S - 1076) + kExpBias;
+  return row_exponent(ab, S) + kExpBias;
 }
 
 // X = round(x * 2^(8S - 2 - E)), |X| <= 2^(8S-1), round half away from zero,
@@ -395,10 +390,11 @@ __device__ __forceinline__ void put_digits(uint64_t y0, uint64_t y1, uint32_t* d
 }
 
 // ---- default split (S = 5): the same 39-bit X as four FP16 digits ----
-// Balanced base-1024 digits a_0..a_3 (a_0 on top), |a_i| <= 512, each stored as
-// an FP16 integer (exact).  With B = 512 (1024^3 + 1024^2 + 1024 + 1), the word
+// Balanced base-1024 digits a_0..a_3 (a_0 on top), each stored as an FP16
+// integer (exact): |a_0| <= 511 by the row's scale (row_exponent), the others in
+// [-512, 511].  With B = 512 (1024^3 + 1024^2 + 1024 + 1), the word
 // Y = 4 (X + B) + 2 bits of fraction holds a_3 + 512, a_2 + 512, a_1 + 512 in
-// bits 2, 12, 22 and a_0 + 512 (up to 1024) from bit 32.
+// bits 2, 12, 22 and a_0 + 512 from bit 32.
 constexpr uint64_t kBias10 = 512ull * ((1ull << 30) + (1ull << 20) + (1ull << 10) + 1ull);
 
 // Y for rows whose k0 >= 66 (every scale above 2^-971), rounded half up: the

@@ -6,9 +6,11 @@ are at their limits so that every partial sum is.
 An entry is rounded to 39 bits below its row's 2^(E+1) and the digit pairs with
 i + j >= 4 are dropped (three of 2^-40 each), so an output is within
 K 2^(Eu+1) 2^(Ev+1) (2 x 2^-40 + 3 x 2^-40) of the exact sum, plus the rounding
-of the diagonals d >= 2 (2^-20 of the products, FP32 sums of at most 512 columns
-between folds: below 2^-38 K of the same scale) and of R (2^-39); 2^-36 K covers
-them all."""
+of the diagonals d >= 2 (2^-20 of the products, FP32 sums of at most 544 columns
+between folds, rounded by 2^5 of 16 x 2^38 a step: below 2^-37 K of the same
+scale) and of R (2^-39); 2^-36 K covers them all.  A row whose largest entry is
+within about 2^-10 below 2^(E+1) is scaled by 2^(E+2) instead, so that no leading
+digit is 512 and the sums of diagonals 0 and 1 stay below 2^24."""
 import numpy as np
 import pytest
 import torch
@@ -31,15 +33,17 @@ def sc():
 def draw(kind, shape, rng):
     if kind == "normal":
         return rng.standard_normal(shape) * 2.0 ** rng.integers(-30, 30, shape[:-1] + (1,))
-    if kind == "largest":      # rounds up to the next power of two: top digits of 512
+    if kind == "largest":      # rounds up to the next power of two at 39 bits: E raised
         return np.full(shape, 2.0 - 2.0 ** -45)
+    if kind == "top":          # the largest that is not raised: leading digits of 511, then 511, 509
+        return np.full(shape, 2.0 - 2.0 ** -9 - 3 * 2.0 ** -20) * (1 - 2.0 ** -36 * rng.integers(0, 2, shape))
     if kind == "aligned":      # every digit 410 in size: all partial sums grow with K
         return np.full(shape, 0.1) * np.where(rng.random(shape[:-1] + (1,)) < 0.5, 1.0, -1.0)
     # lower digits of -512: X = 300 2^30 - 512 (2^20 + 2^10 + 1)
     return np.full(shape, (300 * 2.0 ** 30 - 512 * (2.0 ** 20 + 2.0 ** 10 + 1)) / 2.0 ** 38)
 
 
-@pytest.mark.parametrize("kind", ["normal", "largest", "aligned", "lowest"])
+@pytest.mark.parametrize("kind", ["normal", "largest", "top", "aligned", "lowest"])
 @pytest.mark.parametrize("M,N,K", SIZES)
 def test_digits_and_tiles(sc, M, N, K, kind):
     rng = np.random.default_rng(M + 7 * N + 13 * K)
@@ -50,14 +54,48 @@ def test_digits_and_tiles(sc, M, N, K, kind):
     torch.cuda.synchronize()
     p.check_device_error()
     got = w.cpu().numpy().reshape(M, N)
-    scale = lambda x, axis: 2.0 ** np.ceil(np.log2(np.abs(x).max(axis) * (1 + 2.0 ** -50)))
+    # 2^(E+1), of the raised rows too
+    scale = lambda x, axis: 2.0 ** np.ceil(np.log2(np.abs(x).max(axis) * (1 + 2.0 ** -9)))
     bound = K * 2.0 ** -36 * np.outer(scale(u, 1), scale(v, 0))
     assert np.all(np.abs(got - u @ v) <= bound + 1e-15 * (np.abs(u) @ np.abs(v)))
 
 
-def test_exact_products_at_the_sum_limits(sc):
-    """Entries +-1 and small multiples of 2^-9: two digits each, so every product is
-    in the exact diagonals 0 to 2 and the result is the exact sum."""
+@pytest.mark.parametrize("G,M,N,K", [(1, 130, 70, 128), (1, 130, 70, 2048), (1, 70, 130, 40000),
+                                     (3, 1300, 1172, 96), (3, 1300, 1172, 128), (3, 1300, 1172, 2048),
+                                     (5, 2000, 190, 192), (5, 2000, 190, 2048)])
+def test_one_sign_just_below_a_power_of_two(sc, G, M, N, K):
+    """Integers 1021 and 1023: leading digits of 511 and 512 below their row's own
+    power of two, the second ones -512.  64 products of 512^2 are 2^24, which leaves
+    FP32 no room for the rest of a drain; the sums must be exact (K ranges, wide and
+    narrow tiles)."""
+    rng = np.random.default_rng(K)
+    u = np.full((G, M, K), 1023.0)
+    v = np.full((G, K, N), 1023.0)
+    u[:, :, 0], v[:, 0, :] = 1021.0, 1021.0
+    u[:, ::3, :] -= 2.0 * rng.integers(0, 2, (G, (M + 2) // 3, K))
+    p = sc.Plan("ij,jk->ik", (G,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
+    w = p.contract(torch.from_numpy(u).cuda().reshape(p.shape_u), torch.from_numpy(v).cuda().reshape(p.shape_v))
+    p.check_device_error()
+    assert np.array_equal(w.cpu().numpy().reshape(G, M, N), u @ v)      # |sums| < 2^53
+
+
+@pytest.mark.parametrize("M,N,K", [(96, 80, 1024), (300, 260, 1024), (64, 72, 9000)])
+def test_entries_near_one_from_below(sc, M, N, K):
+    """cos of small angles: nine leading digits in ten would be 512 at the row's own
+    power of two.  Within the split form's 1e-10 in the 2-norm, 1e-9 at most."""
+    rng = np.random.default_rng(M)
+    u, v = np.cos(0.02 * rng.standard_normal((M, K))), np.cos(0.02 * rng.standard_normal((K, N)))
+    p = sc.Plan("ij,jk->ik", (1,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
+    w = p.contract(torch.from_numpy(u).cuda().reshape(p.shape_u), torch.from_numpy(v).cuda().reshape(p.shape_v))
+    e = w.cpu().numpy().reshape(M, N) - u @ v
+    assert np.linalg.norm(e) <= 1e-10 * np.linalg.norm(u @ v)
+    assert np.all(np.abs(e) <= 1e-9 * (u @ v))
+
+
+def test_exact_products_of_either_sign(sc):
+    """Entries +-1 (leading digit 256) and small multiples of 2^-9: two digits each, so
+    every product is in diagonals 0 to 2, whose sums here are integers that FP32 holds,
+    and the result is the exact sum."""
     rng = np.random.default_rng(3)
     M, N, K = 130, 70, 20000
     u, v = (rng.choice([1.0, -1.0, 2.0 ** -9, 3.0 * 2.0 ** -9], (r, K)) for r in (M, N))

@@ -6,8 +6,16 @@ round to nearest even like the kernel's.
   integer round(y) (ties to even) in its low mantissa bits.
 * The final drain's round(acc3 * 2^24) for |acc3| < 64: h = round(acc3 * 2^16)
   by the magic number, the remainder acc3 - h 2^-16 exact in FP32, and
-  round(acc3 * 2^24) = 2^8 h + round(remainder * 2^24)."""
+  round(acc3 * 2^24) = 2^8 h + round(remainder * 2^24).
+* The default split's row scale and digits (tests/native, compiled with the host
+  compiler against the library's internal header): no leading digit above 511, and
+  the sums between two drains below 2^24."""
+import os
+import shutil
+import subprocess
+
 import numpy as np
+import pytest
 
 F = np.float32
 M0 = F(12582912.0)  # 1.5 * 2^23
@@ -57,3 +65,21 @@ def test_drain_bound_fits_the_magic_window():
     |a_i b_j| <= 2^14 (diagonals 2, 1, 0), so the FP32 sum is an integer
     within the magic-number window 2^22."""
     assert max(3 * 64, 2 * 128, 1 * 256) * 2 ** 14 <= 2 ** 22
+
+
+def test_row_scale_keeps_the_leading_digit_below_512(tmp_path):
+    here = os.path.dirname(os.path.abspath(__file__))
+    root = os.path.dirname(here)
+    cxx = shutil.which("g++")
+    inc = next((os.path.join(d, "include") for d in (os.environ.get("CUDA_HOME"), "/usr/local/cuda")
+                if d and os.path.exists(os.path.join(d, "include", "cuda_runtime.h"))), None)
+    if not cxx or not inc:
+        pytest.skip("needs g++ and the CUDA runtime headers")
+    exe = str(tmp_path / "split_digits_check")
+    subprocess.run([cxx, "-O2", "-std=c++17", "-I", os.path.join(root, "include"), "-I",
+                    os.path.join(root, "paper_2007_08056_gb300", "csrc"), "-I", inc,
+                    os.path.join(here, "native", "split_digits_check.cpp"), "-o", exe],
+                   check=True, capture_output=True, text=True)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert r.stdout.startswith("ok ")
