@@ -63,15 +63,17 @@ def test_digits_and_tiles(sc, M, N, K, kind):
 @pytest.mark.parametrize("G,M,N,K", [(1, 130, 70, 128), (1, 130, 70, 2048), (1, 70, 130, 40000),
                                      (3, 1300, 1172, 96), (3, 1300, 1172, 128), (3, 1300, 1172, 2048),
                                      (5, 2000, 190, 192), (5, 2000, 190, 2048)])
-def test_one_sign_just_below_a_power_of_two(sc, G, M, N, K):
+@pytest.mark.parametrize("top", [1023.0, 1021.0])
+def test_one_sign_just_below_a_power_of_two(sc, G, M, N, K, top):
     """Integers 1021 and 1023: leading digits of 511 and 512 below their row's own
     power of two, the second ones -512.  64 products of 512^2 are 2^24, which leaves
-    FP32 no room for the rest of a drain; the sums must be exact (K ranges, wide and
-    narrow tiles)."""
+    FP32 no room for the rest of a drain, so rows with 1023 are raised; 1019 and 1021
+    are not: 64 x 511^2 and 64 x 511 x 512 are the most that diagonals 0 and 1 hold.
+    The sums must be exact (K ranges, wide and narrow tiles)."""
     rng = np.random.default_rng(K)
-    u = np.full((G, M, K), 1023.0)
-    v = np.full((G, K, N), 1023.0)
-    u[:, :, 0], v[:, 0, :] = 1021.0, 1021.0
+    u = np.full((G, M, K), top)
+    v = np.full((G, K, N), top)
+    u[:, :, 0], v[:, 0, :] = top - 2.0, top - 2.0
     u[:, ::3, :] -= 2.0 * rng.integers(0, 2, (G, (M + 2) // 3, K))
     p = sc.Plan("ij,jk->ik", (G,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "split_bf16")
     w = p.contract(torch.from_numpy(u).cuda().reshape(p.shape_u), torch.from_numpy(v).cuda().reshape(p.shape_v))
