@@ -339,12 +339,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tma_load_4d(&tma_b, &full[st], sb, kc, (int)n0, b);
         ++issued;
       }
-      if (ctl->abort) {
-        // let the copies this thread issued land before the CTA exits
-        int first = issued > STAGES ? issued - STAGES : 0;
-        for (int kb = first; kb < issued; ++kb)
-          wait_phase(&full[kb % STAGES], (kb / STAGES) & 1, ctl, kTimeoutCycles / 2);
-      }
+      // the last copies land before the CTA exits
+      for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
+        wait_landed(&full[kb % STAGES], (kb / STAGES) & 1, ctl);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -393,7 +390,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
       tc_commit(acc_full);
       tc_commit(drain);
-      wait_phase(drain, 0, ctl, kTimeoutCycles / 2);
+      wait_landed(drain, 0, ctl);
     }
   } else if (warp >= EPI_WARP0) {
     // ------------------------------------------------------------ epilogue

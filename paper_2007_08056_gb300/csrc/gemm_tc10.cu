@@ -89,7 +89,7 @@ struct Cfg {
   static_assert(REGION >= STAGING, "the epilogue staging fits the stages");
   static constexpr int FIRST = STAGES - 1;
   static constexpr bool EARLY = (size_t)FIRST * STAGE_BYTES >= STAGING;   // loads beside the epilogue
-  static constexpr int BARS = 2 * STAGES + 7;
+  static constexpr int BARS = 2 * STAGES + 9;
   static constexpr int TAB = 12 * (TN + TM);      // offsets and exponents of a tile
   static constexpr size_t SMEM = REGION + 8 * BARS + 2 * TAB + 16 + 64;
 };
@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
   uint64_t* acc_full = drained + 2;      // a tile's MMAs are done
   uint64_t* zero_done = acc_full + 1;    // its accumulators are read out and zeroed
   uint64_t* staged = zero_done + 1;      // its results have left the staging
-  uint8_t* tabs = (uint8_t*)(staged + 1);      // [2] tables of this tile and the last one
+  uint64_t* issued = staged + 1;         // [2] all of an issuing thread's MMAs are done
+  uint8_t* tabs = (uint8_t*)(issued + 2);      // [2] tables of this tile and the last one
   uint32_t* tmem_slot = (uint32_t*)(tabs + 2 * C::TAB);
   Ctl* ctl = (Ctl*)(tmem_slot + 4);
 
@@ -255,6 +256,7 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
     for (int h = 0; h < 2; ++h) {
       mbar_init(&go[h], 1);
       mbar_init(&drained[h], 8);
+      mbar_init(&issued[h], 1);
     }
     mbar_init(acc_full, H);
     mbar_init(zero_done, 8 * H);
@@ -313,11 +315,9 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
           st = st + 1 == STAGES ? 0 : st + 1;
         }
       }
-      if (ctl->abort) {
-        // let the copies this thread issued land before the CTA exits
-        for (int s = 0; s < STAGES; ++s)
-          if ((live >> s) & 1) wait_phase(&full[s], ((ph >> s) & 1) ^ 1, ctl, kTimeoutCycles / 2);
-      }
+      // the last copies land before the CTA exits
+      for (int s = 0; s < STAGES; ++s)
+        if ((live >> s) & 1) wait_landed(&full[s], ((ph >> s) & 1) ^ 1, ctl);
     }
   } else if (warp <= H) {
     // ------------------------------------------------------------ MMA issuers
@@ -367,9 +367,10 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
           st = st + 1 == STAGES ? 0 : st + 1;
         }
         tc_commit(acc_full);
-        // (keeps the MMAs in flight from outliving the CTA after an abort)
-        if (!ok) wait_phase(acc_full, it & 1, ctl, kTimeoutCycles / 2);
       }
+      // the last MMAs are done before the CTA gives its TMEM back, after an abort too
+      tc_commit(&issued[h]);
+      wait_landed(&issued[h], 0, ctl);
     }
   } else if (warp >= EPI_WARP0) {
     // ------------------------------------------------------------ epilogue

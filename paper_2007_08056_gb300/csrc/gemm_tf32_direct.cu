@@ -173,10 +173,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         for (int i = 0; i < NB; ++i) tma_load_4d(&tma_b, &b_full[st], sb + i * B_BYTES, kb * KST, i * BH, b);
         ++issued;
       }
-      if (ctl->abort) {
-        for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-          wait_phase(&b_full[kb % STAGES], (kb / STAGES) & 1, ctl, kTimeoutCycles / 2);
-      }
+      // the last copies land before the CTA exits
+      for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
+        wait_landed(&b_full[kb % STAGES], (kb / STAGES) & 1, ctl);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -205,7 +204,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tc_commit(&empty[st]);
       }
       tc_commit(acc_full);
-      wait_phase(acc_full, 0, ctl, kTimeoutCycles / 2);
+      wait_landed(acc_full, 0, ctl);
     }
   } else if (warp >= W0) {
     // ------------------------------------------------------------ long operand

@@ -92,6 +92,22 @@ __device__ __forceinline__ bool wait_phase_sleep(uint64_t* bar, uint32_t parity,
   }
 }
 
+// Before a CTA leaves: wait for its own copies or MMAs in flight, after an abort
+// too (the waits above give up at once then), so that none writes to shared
+// memory or TMEM that the next CTA holds.  Bounded by the limit alone.
+__device__ __forceinline__ bool wait_landed(uint64_t* bar, uint32_t parity, Ctl* ctl,
+                                            long long limit = kTimeoutCycles / 2) {
+  const long long t0 = clock64();
+  while (!mbar_test_sleep(bar, parity)) {
+    if (clock64() - t0 > limit) {
+      atomicOr(ctl->err, (unsigned)DEVERR_TIMEOUT);
+      ctl->abort = 1;
+      return false;
+    }
+  }
+  return true;
+}
+
 // Box of a [planes][batches][rows][k] map at (k = c0, row = c1, batch = c2, plane 0).
 __device__ __forceinline__ void tma_load_4d(const CUtensorMap* map, uint64_t* bar, void* dst, int c0, int c1,
                                             int c2) {

@@ -1,7 +1,11 @@
 """Failure detection without a GPU fault: a kernel whose bounded wait runs out
 (on a barrier that nothing completes) records the timeout in the workspace's
 error word and returns; the host reads the status, and the context goes on
-to run a correct contraction."""
+to run a correct contraction.  Copies and MMAs in flight are waited for before a
+CTA leaves, after an abort too."""
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -49,3 +53,15 @@ def test_selftest_argument_errors(sc):
     with pytest.raises(sc.SymctrError) as ei:
         sc.selftest_bounded_wait(small)
     assert ei.value.status == 7           # SYMCTR_ERR_WORKSPACE
+
+
+def test_copies_in_flight_are_waited_for_after_an_abort(sc, tmp_path):
+    from paper_2007_08056_gb300 import build as B
+
+    exe = str(tmp_path / "landed_check")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native", "landed_check.cu")
+    r = subprocess.run([B.nvcc()] + B._flags() + [src, "-o", exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert r.stdout == "ok\n"
