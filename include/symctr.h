@@ -297,13 +297,19 @@ SYMCTR_API symctr_status symctr_contract(const symctr_plan* plan, const double* 
  * plan's precision form on the real and imaginary parts (four times the real
  * work), with the same workspace and error reporting as symctr_contract.  The
  * default split form prepares each part once, in two GEMM launches, when the
- * workspace holds both parts: 2 workspace_bytes + 16 n_q M N + 256 n_q (M + N) +
- * 4096 bytes do.
+ * workspace holds both parts (symctr_plan_workspace_bytes_complex).
  * Returns as symctr_contract. */
 SYMCTR_API symctr_status symctr_contract_complex(const symctr_plan* plan, int conj_u, int conj_v,
                                                 const double* u_red, const double* v_red,
                                                 double* w_red, void* workspace,
                                                 size_t workspace_bytes, void* stream);
+
+/* Device workspace with which symctr_contract_complex prepares each part of the
+ * operands once (at most 2 workspace_bytes + 16 n_q M N + 256 n_q (M + N) + 4096);
+ * workspace_bytes where it never does: any form but the default split form on
+ * the tensor cores (n_slices = 5, symctr_plan_info.tensor_core = 1).  0 for NULL.
+ * Host only. */
+SYMCTR_API uint64_t symctr_plan_workspace_bytes_complex(const symctr_plan* plan);
 
 /* symctr_contract without a caller-provided workspace, for callers that cannot
  * allocate device memory (they are handed only their input and output buffers,

@@ -122,6 +122,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.symctr_selftest_bounded_wait.argtypes = [P, ctypes.c_size_t, ctypes.c_int64, P]
     lib.symctr_contract_complex.argtypes = [P, ctypes.c_int, ctypes.c_int, P, P, P, P,
                                             ctypes.c_size_t, P]
+    lib.symctr_plan_workspace_bytes_complex.argtypes = [P]
+    lib.symctr_plan_workspace_bytes_complex.restype = ctypes.c_uint64
     lib.symctr_plan_attach_tables.argtypes = [P, P, ctypes.c_size_t, P]
     lib.symctr_plan_chain.argtypes = [P, P, P, ctypes.c_int]
     lib.symctr_plan_destroy.argtypes = [P]
@@ -272,7 +274,7 @@ class Plan:
         self.shape_u, self.shape_v, self.shape_w = shape(su), shape(sv), shape(self.sym_w)
         self._size_u, self._size_v, self._size_w = (torch.Size(self.shape_u), torch.Size(self.shape_v),
                                                      torch.Size(self.shape_w))
-        self._ws = None
+        self._ws = self._outgrown = None
         self._tables = None
         self._tables_ready = info.table_bytes == 0
         self._lock = threading.Lock()
@@ -365,12 +367,13 @@ class Plan:
 
     def _workspace_complex(self, device) -> torch.Tensor:
         """The plan's workspace, grown to hold both parts of complex operands (each
-        part is then prepared once) where that takes at most 2 GiB."""
-        i = self.info
-        M, N, n_q = int(i.M), int(i.N), int(i.n_q)
-        need = 2 * int(i.workspace_bytes) + 16 * n_q * M * N + 256 * n_q * (M + N) + 4096
-        if need <= 2 << 30 and (self._ws is None or self._ws.numel() < need):
-            self._ws = torch.empty(need, dtype=torch.uint8, device=device or "cuda")
+        part is then prepared once) where that takes at most 2 GiB and the plan's
+        form does so.  A smaller one that this replaces lives as long as the plan: a
+        captured graph of earlier calls still works in it."""
+        need = int(load().symctr_plan_workspace_bytes_complex(self._h))
+        if int(self.info.workspace_bytes) < need <= 2 << 30 and (self._ws is None or self._ws.numel() < need):
+            grown = torch.empty(need, dtype=torch.uint8, device=device or "cuda")
+            self._outgrown, self._ws = self._ws, grown
             self._seen = set()
         return self.workspace(device=device)
 

@@ -1301,7 +1301,7 @@ static bool chain_sides(const symctr_plan* src, const std::vector<int>& rows,
 // of four.  Returns false when the workspace is too small or the plan does not
 // run this form; the caller then takes the parts one product at a time.
 static bool complex_layout(const symctr_plan* P, uint64_t ws_bytes, Layout* L, int64_t* acc_n) {
-  if (!P->tensor_core || P->prec != SYMCTR_SPLIT_BF16 || P->n_slices != 5) return false;
+  if (!P->tensor_core || P->prec != SYMCTR_SPLIT_BF16 || P->n_slices != 5 || P->run.n_q < 1) return false;
   Problem both = P->run;
   both.n_q *= 2;   // real and imaginary parts as batches
   *L = make_layout(both, true, P->general, P->prec, P->n_slices, P->kpad);
@@ -1408,6 +1408,13 @@ symctr_status symctr_plan_create_general(const char* einsum, int n_moduli, const
   dv.sector_dims = v->sector_dims;
   return build(einsum, n_moduli, moduli, du, dv, signs_w_or_null, charge_w_or_null, prec, n_slices,
                true, out);
+}
+
+uint64_t symctr_plan_workspace_bytes_complex(const symctr_plan* P) {
+  if (!P) return 0;
+  Layout both;
+  int64_t acc_n = 0;
+  return complex_layout(P, UINT64_MAX, &both, &acc_n) ? both.bytes : P->ws_bytes;
 }
 
 symctr_status symctr_plan_query(const symctr_plan* P, symctr_plan_info* o) {
@@ -1568,7 +1575,7 @@ symctr_status symctr_contract_complex(const symctr_plan* P, int conj_u, int conj
   const double su = conj_u ? -1.0 : 1.0, sv = conj_v ? -1.0 : 1.0;
   Layout both;
   int64_t acc_n = 0;
-  if (ws && P->run.n_q > 0 && complex_layout(P, ws_bytes, &both, &acc_n))
+  if (ws && complex_layout(P, ws_bytes, &both, &acc_n))
     return run_complex_split(P, su < 0 ? -1 : 1, sv < 0 ? -1 : 1, u, v, w, ws, both, acc_n, st);
   // (Ur + i su Ui)(Vr + i sv Vi) = Ur Vr - su sv Ui Vi + i (sv Ur Vi + su Ui Vr):
   // four real contractions on the real (+0) and imaginary (+1) parts

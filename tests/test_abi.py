@@ -124,6 +124,40 @@ def test_null_arguments():
     assert lib.symctr_selftest_bounded_wait(None, 0, 0, None) == 6
 
 
+def complex_bytes(p):
+    i = p.info
+    need = int(sc.load().symctr_plan_workspace_bytes_complex(p._h))
+    most = 2 * i.workspace_bytes + 16 * i.n_q * i.M * i.N + 256 * i.n_q * (i.M + i.N) + 4096
+    return need, most
+
+
+def test_workspace_of_complex_contractions():
+    """Only the default split form on the tensor cores prepares both parts at once: no
+    other plan asks for more than its own workspace, and the binding allocates what
+    is asked for.  A workspace that it outgrows lives on (captured graphs)."""
+    assert sc.load().symctr_plan_workspace_bytes_complex(None) == 0
+    su, sv = ((1, -1), (0,), (40, 40)), ((1, 1, -1), (0,), (40, 2, 40))
+    for prec, slices in (("fp64", 0), ("tf32", 0), ("split_bf16", 3), ("split_bf16", 6)):
+        p = sc.Plan(WL.MPS_STEP1, (3,), su, sv, prec, n_slices=slices)
+        assert complex_bytes(p)[0] == p.info.workspace_bytes
+        assert p._workspace_complex("cpu").numel() == max(p.info.workspace_bytes, 256)
+    peps = sc.Plan(WL.PEPS_Y, WL.PEPS_MODULI, (WL.PEPS_T.signs, (0, 0), (4,) * 4 + (2,)),
+                   (WL.PEPS_ENV.signs, (0, 0), (4,) * 4), "split_bf16")
+    assert peps.info.tensor_core == 0 and complex_bytes(peps)[0] == peps.info.workspace_bytes
+    p = sc.Plan(WL.MPS_STEP1, (3,), su, sv, "split_bf16")
+    need, most = complex_bytes(p)
+    assert p.info.workspace_bytes < need <= most
+    small = p.workspace(device="cpu")
+    assert p._workspace_complex("cpu").numel() == need and p._outgrown is small
+    assert p.workspace(device="cpu").numel() == need
+    # a general plan: the sizes that run, not the whole ones
+    sizes = (40, 3, 3)
+    g = sc.Plan(WL.MPS_STEP1, (3,), ((1, -1), (0,), (40, 40), (3, 3), (sizes, sizes)),
+                ((1, 1, -1), (0,), (40, 40, 40), (3, 3, 3), (sizes,) * 3), "split_bf16")
+    need, _ = complex_bytes(g)
+    assert g.info.workspace_bytes < need < 2 * g.info.workspace_bytes + 16 * g.info.n_q * g.info.M * g.info.N
+
+
 def test_workspace_too_small_is_rejected_before_any_launch():
     """The size check happens on the host, so it needs no GPU."""
     p = sc.Plan(WL.Z3_ORDER4.einsum, (3,), (WL.PP, (0,), (4,) * 4), (WL.PP, (0,), (4,) * 4),

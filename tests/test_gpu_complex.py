@@ -114,3 +114,29 @@ def test_both_parts_at_once(sc, dims, conj):
             p.check_device_error(ws)
             assert rel(w.cpu().numpy().real, want.real) <= TOL["split_bf16"]
             assert rel(w.cpu().numpy().imag, want.imag) <= TOL["split_bf16"]
+
+
+def test_captured_graph_outlives_a_grown_workspace(sc):
+    """A graph of real contractions, captured before a complex contraction makes the
+    plan's workspace grow, still works in the workspace it was captured with: what is
+    allocated afterwards keeps its contents, and the replayed result is the same."""
+    G, bond, phys = 4, 64, 2
+    su, sv = ((1, -1), (0,), (bond, bond)), ((1, 1, -1), (0,), (bond, phys, bond))
+    p = sc.Plan("ab,asg->bsg", (G,), su, sv, "split_bf16")
+    u, v = (torch.from_numpy(cdraw((G,), s, 41)).cuda() for s in (su, sv))
+    ur, vr = u.real.contiguous(), v.real.contiguous()
+    want = p.contract(ur, vr)
+    w = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        p.contract(ur, vr, out=w)
+    size = p.workspace().numel()
+    p.contract_complex(u, v)
+    assert p.workspace().numel() > size
+    later = [torch.full((size,), 7, dtype=torch.uint8, device="cuda") for _ in range(4)]
+    g.replay()
+    torch.cuda.synchronize()
+    p.check_device_error()
+    assert torch.equal(w, want)
+    assert all(int((t != 7).sum()) == 0 for t in later)
