@@ -36,141 +36,195 @@ __host__ __device__ inline bool map_rows_fast(const AxisMap& rows) {
   return rows.n > 0 && rows.bstride[rows.n - 1] == 1;
 }
 
-// GEMM-shaped problems, T x T output tiles by 256 threads: (T / 16)^2 outputs a
+// GEMM-shaped problems, a T x T output tile by 256 threads: (T / 16)^2 outputs a
 // thread, or (T = 8) one output by four threads that split each K block.  The
 // float64 pipe (2 FMAs per SM and clock) is the bound at every T: what matters
 // is that all SMs have the same share, and that a small problem has tiles for
 // all of them (tile_choice): 48 x 48 x 48 by 3 irreps ran on three SMs with
 // 64 x 64 tiles, 65 -> 17 us (launch-bound) with 8 x 8; the two MPS contractions
-// 128 x 2048 x 128 and 128 x 128 x 2048 by 8 irreps, on 3.4 tiles per SM and on
-// 128 of 152 SMs, 1177 -> 951 us with 32 x 32 and 7 K ranges (909 us at the
-// float64 rate of a large product).  Column offsets are computed for kKc columns of K
-// at a time, one per thread; the next K block's gathers are in flight while
-// this one is multiplied.
+// 128 x 2048 x 128 and 128 x 128 x 2048 by 8 irreps, on 3.4 such tiles per SM and
+// on 128 of 152 SMs, 1177 -> 922 us with 16 x 16 (909 us at the float64 rate of a
+// large product).  Column offsets are computed for kKc columns of K at a time,
+// one per thread; the next K block's gathers are in flight while this one is
+// multiplied.  One CTA to a tile and range: a grid of four CTAs per SM walking
+// them left SMs with one more or less than their share (640 x 640 x 2000 by 2
+// irreps in 16 x 16 tiles 3316 us, 2781 without the walk).
+// The K ranges of a tile are the CTAs of a cluster: each leaves its partial sums in
+// shared memory, and every CTA adds up a share of the tile over the ranks, in their
+// order, and writes it, so that a product repeats bit for bit.  (Float64 atomics
+// onto a zeroed W, 475 us for the second MPS contraction against 473, gave
+// results of three and more ranges that differed from run to run.)
 // General plans pass their offset tables (t.urow != NULL): offsets come from
 // them, -1 marking an absent aligned row or column (read as zero, not stored).
 constexpr int kKc = 256;
+constexpr int kMaxRanges = 16;    // CTAs of a cluster
+
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The float64 word of cluster CTA `rank` at this CTA's shared address of it.
+__device__ __forceinline__ double cluster_ld(const double* p, int rank) {
+  double x;
+  asm volatile(
+      "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %1, %2;\n\t"
+      "ld.shared::cluster.f64 %0, [ra];\n\t}\n"
+      : "=d"(x)
+      : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank)
+      : "memory");
+  return x;
+}
 
 template <int T>
-__global__ void __launch_bounds__(THREADS) gemm_f64_tiled(const __grid_constant__ Problem p, int ksplit,
-                                                          int64_t kchunk, bool u_rows_fast, bool v_rows_fast,
-                                                          const Tables t, const double* __restrict__ U,
-                                                          const double* __restrict__ V, double* __restrict__ W) {
+__global__ void __launch_bounds__(THREADS, T == 64 ? 2 : T == 32 ? 3 : 4)
+    gemm_f64_tiled(const __grid_constant__ Problem p, int ksplit, int64_t kchunk, bool u_rows_fast, bool v_rows_fast,
+                   const Tables t, const double* __restrict__ U, const double* __restrict__ V, double* __restrict__ W) {
   constexpr int R = T >= 16 ? T / 16 : 1;                      // outputs per thread and side
   constexpr int NL = (T * BK + THREADS - 1) / THREADS;         // gathers per thread, operand and K block
-  __shared__ double As[2][BK][T + 1];
-  __shared__ double Bs[2][BK][T + 1];
+  __shared__ double ops[2][2][BK][T + 1];
+  double (*As)[BK][T + 1] = ops[0];
+  double (*Bs)[BK][T + 1] = ops[1];
   __shared__ int64_t uoff[T], voff[T], woffr[T], woffc[T], ku[kKc], kv[kKc];
   const int tid = threadIdx.x;
   const int tr = T >= 16 ? tid / 16 : (tid & 63) / 8, tc = T >= 16 ? tid % 16 : tid % 8;
   const int64_t mt = (p.M + T - 1) / T, nt = (p.N + T - 1) / T;
-  const int64_t ntiles = mt * nt * p.n_q * ksplit;
   const bool tab = t.urow != nullptr;
-  for (int64_t tI = blockIdx.x; tI < ntiles; tI += gridDim.x) {
-    const int64_t ks = tI % ksplit;
-    const int64_t t2 = tI / ksplit;
-    const int64_t b = t2 / (mt * nt);
-    const int64_t rem = t2 - b * mt * nt;
-    const int64_t m0 = (rem / nt) * T, n0 = (rem % nt) * T;
-    const int Q = batch_irrep(p, (int)b);
-    const int64_t kbeg = ks * kchunk, kend = kbeg + kchunk < p.K ? kbeg + kchunk : p.K;
-    __syncthreads();
-    if (tid < T) {
-      const int64_t m = m0 + tid;
-      uoff[tid] = m >= p.M ? -1 : tab ? t.urow[b * p.M + m] : aoff(p.u.rows, p.g, Q, m);
-      woffr[tid] = m >= p.M ? -1 : tab ? t.wrow[b * p.M + m] : aoff(p.w.rows, p.g, Q, m);
-    } else if (tid >= 128 && tid < 128 + T) {
-      const int64_t n = n0 + tid - 128;
-      voff[tid - 128] = n >= p.N ? -1 : tab ? t.vrow[b * p.N + n] : aoff(p.v.rows, p.g, Q, n);
-      woffc[tid - 128] = n >= p.N ? -1 : tab ? t.wcol[b * p.N + n] : aoff(p.w.cols, p.g, Q, n);
-    }
-    double acc[R][R];
+  const int ks = (int)(blockIdx.x % (unsigned)ksplit);   // K range, rank in the cluster
+  const int64_t t2 = blockIdx.x / (unsigned)ksplit;
+  const int64_t b = t2 / (mt * nt);
+  const int64_t rem = t2 - b * mt * nt;
+  const int64_t m0 = (rem / nt) * T, n0 = (rem % nt) * T;
+  const int Q = batch_irrep(p, (int)b);
+  const int64_t kbeg = ks * kchunk, kend = kbeg + kchunk < p.K ? kbeg + kchunk : p.K;
+  if (tid < T) {
+    const int64_t m = m0 + tid;
+    uoff[tid] = m >= p.M ? -1 : tab ? t.urow[b * p.M + m] : aoff(p.u.rows, p.g, Q, m);
+    woffr[tid] = m >= p.M ? -1 : tab ? t.wrow[b * p.M + m] : aoff(p.w.rows, p.g, Q, m);
+  } else if (tid >= 128 && tid < 128 + T) {
+    const int64_t n = n0 + tid - 128;
+    voff[tid - 128] = n >= p.N ? -1 : tab ? t.vrow[b * p.N + n] : aoff(p.v.rows, p.g, Q, n);
+    woffc[tid - 128] = n >= p.N ? -1 : tab ? t.wcol[b * p.N + n] : aoff(p.w.cols, p.g, Q, n);
+  }
+  // the sum of each kKc columns, and their sum: shorter chains of roundings
+  double acc[R][R], sum[R][R];
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int j = 0; j < R; ++j) sum[i][j] = 0.0;
+  for (int64_t kc = kbeg; kc < kend; kc += kKc) {
 #pragma unroll
     for (int i = 0; i < R; ++i)
 #pragma unroll
       for (int j = 0; j < R; ++j) acc[i][j] = 0.0;
-    for (int64_t kc = kbeg; kc < kend; kc += kKc) {
-      const int n = kend - kc < kKc ? (int)(kend - kc) : kKc;
-      __syncthreads();
-      if (tid < n) {
-        const int64_t k = kc + tid;
-        ku[tid] = tab ? t.ucol[b * p.K + k] : aoff(p.u.cols, p.g, Q, k);
-        kv[tid] = tab ? t.vcol[b * p.K + k] : aoff(p.v.cols, p.g, Q, k);
-      }
-      __syncthreads();
-      double xa[NL], xb[NL];
-      auto gather = [&](int k0) {
-#pragma unroll
-        for (int j = 0; j < NL; ++j) {
-          const int e = tid + j * THREADS;
-          xa[j] = xb[j] = 0.0;
-          if (e < T * BK) {
-            int mm = u_rows_fast ? e % T : e / BK, kk = k0 + (u_rows_fast ? e / T : e % BK);
-            if (kk < n && uoff[mm] >= 0 && ku[kk] >= 0) xa[j] = U[p.es * (uoff[mm] + ku[kk])];
-            mm = v_rows_fast ? e % T : e / BK, kk = k0 + (v_rows_fast ? e / T : e % BK);
-            if (kk < n && voff[mm] >= 0 && kv[kk] >= 0) xb[j] = V[p.es * (voff[mm] + kv[kk])];
-          }
-        }
-      };
-      auto stage = [&](int buf) {
-#pragma unroll
-        for (int j = 0; j < NL; ++j) {
-          const int e = tid + j * THREADS;
-          if (e < T * BK) {
-            As[buf][u_rows_fast ? e / T : e % BK][u_rows_fast ? e % T : e / BK] = xa[j];
-            Bs[buf][v_rows_fast ? e / T : e % BK][v_rows_fast ? e % T : e / BK] = xb[j];
-          }
-        }
-      };
-      gather(0);
-      stage(0);
-      __syncthreads();
-      for (int k0 = 0, buf = 0; k0 < n; k0 += BK, buf ^= 1) {
-        if (k0 + BK < n) gather(k0 + BK);
-        if constexpr (T >= 16) {
-#pragma unroll
-          for (int kk = 0; kk < BK; ++kk) {
-            double a[R], bb[R];
-#pragma unroll
-            for (int i = 0; i < R; ++i) a[i] = As[buf][kk][tr + 16 * i];
-#pragma unroll
-            for (int j = 0; j < R; ++j) bb[j] = Bs[buf][kk][tc + 16 * j];
-#pragma unroll
-            for (int i = 0; i < R; ++i)
-#pragma unroll
-              for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
-          }
-        } else {
-#pragma unroll
-          for (int q = 0; q < BK / 4; ++q) {
-            const int kk = (tid >> 6) * (BK / 4) + q;
-            acc[0][0] = fma(As[buf][kk][tr], Bs[buf][kk][tc], acc[0][0]);
-          }
-        }
-        if (k0 + BK < n) stage(buf ^ 1);
-        __syncthreads();
-      }
+    const int n = kend - kc < kKc ? (int)(kend - kc) : kKc;
+    __syncthreads();
+    if (tid < n) {
+      const int64_t k = kc + tid;
+      ku[tid] = tab ? t.ucol[b * p.K + k] : aoff(p.u.cols, p.g, Q, k);
+      kv[tid] = tab ? t.vcol[b * p.K + k] : aoff(p.v.cols, p.g, Q, k);
     }
-    if constexpr (T < 16) {
-      double* red = &As[0][0][0];
-      static_assert(T >= 16 || sizeof(As) >= THREADS * sizeof(double), "reduction buffer");
-      red[tid] = acc[0][0];
+    __syncthreads();
+    double xa[NL], xb[NL];
+    auto gather = [&](int k0) {
+#pragma unroll
+      for (int j = 0; j < NL; ++j) {
+        const int e = tid + j * THREADS;
+        xa[j] = xb[j] = 0.0;
+        if (e < T * BK) {
+          int mm = u_rows_fast ? e % T : e / BK, kk = k0 + (u_rows_fast ? e / T : e % BK);
+          if (kk < n && uoff[mm] >= 0 && ku[kk] >= 0) xa[j] = U[p.es * (uoff[mm] + ku[kk])];
+          mm = v_rows_fast ? e % T : e / BK, kk = k0 + (v_rows_fast ? e / T : e % BK);
+          if (kk < n && voff[mm] >= 0 && kv[kk] >= 0) xb[j] = V[p.es * (voff[mm] + kv[kk])];
+        }
+      }
+    };
+    auto stage = [&](int buf) {
+#pragma unroll
+      for (int j = 0; j < NL; ++j) {
+        const int e = tid + j * THREADS;
+        if (e < T * BK) {
+          As[buf][u_rows_fast ? e / T : e % BK][u_rows_fast ? e % T : e / BK] = xa[j];
+          Bs[buf][v_rows_fast ? e / T : e % BK][v_rows_fast ? e % T : e / BK] = xb[j];
+        }
+      }
+    };
+    gather(0);
+    stage(0);
+    __syncthreads();
+    for (int k0 = 0, buf = 0; k0 < n; k0 += BK, buf ^= 1) {
+      if (k0 + BK < n) gather(k0 + BK);
+      if constexpr (T >= 16) {
+#pragma unroll
+        for (int kk = 0; kk < BK; ++kk) {
+          double a[R], bb[R];
+#pragma unroll
+          for (int i = 0; i < R; ++i) a[i] = As[buf][kk][tr + 16 * i];
+#pragma unroll
+          for (int j = 0; j < R; ++j) bb[j] = Bs[buf][kk][tc + 16 * j];
+#pragma unroll
+          for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < BK / 4; ++q) {
+          const int kk = (tid >> 6) * (BK / 4) + q;
+          acc[0][0] = fma(As[buf][kk][tr], Bs[buf][kk][tc], acc[0][0]);
+        }
+      }
+      if (k0 + BK < n) stage(buf ^ 1);
       __syncthreads();
-      if (tid < 64) acc[0][0] = (red[tid] + red[tid + 64]) + (red[tid + 128] + red[tid + 192]);
-      if (tid >= 64) continue;
     }
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int mm = tr + 16 * i;
-      if (woffr[mm] < 0) continue;
+    for (int i = 0; i < R; ++i)
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const int nn = tc + 16 * j;
-        if (woffc[nn] < 0) continue;
-        double* dst = W + p.es * (woffr[mm] + woffc[nn]);
-        if (ksplit > 1) atomicAdd(dst, signed_result(p, acc[i][j]));
-        else store_w(p, dst, acc[i][j]);
+      for (int j = 0; j < R; ++j) sum[i][j] += acc[i][j];
+  }
+  double* part = &ops[0][0][0][0];   // [T][T] partial sums, in place of the operands
+  if constexpr (T < 16) {
+    double* red = part;
+    part += THREADS;
+    red[tid] = sum[0][0];
+    __syncthreads();
+    if (tid < 64) sum[0][0] = (red[tid] + red[tid + 64]) + (red[tid + 128] + red[tid + 192]);
+  }
+  static_assert(sizeof(ops) >= (T * T + (T < 16 ? THREADS : 0)) * sizeof(double), "partial sums");
+  if (ksplit > 1) {
+    if (T >= 16 || tid < 64) {
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) part[(tr + 16 * i) * T + tc + 16 * j] = sum[i][j];
+    }
+    cluster_sync_all();
+    for (int e = ks * THREADS + tid; e < T * T; e += ksplit * THREADS) {
+      const int64_t ro = woffr[e / T], co = woffc[e % T];
+      if (ro < 0 || co < 0) continue;
+      double x = 0.0;
+      for (int r0 = 0; r0 < ksplit; r0 += 4) {
+        double y[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) y[r] = r0 + r < ksplit ? cluster_ld(part + e, r0 + r) : 0.0;
+        x += y[0];
+        x += y[1];
+        x += y[2];
+        x += y[3];
       }
+      store_w(p, W + p.es * (ro + co), x);
+    }
+    cluster_sync_all();   // the others have read this CTA's sums
+    return;
+  }
+  if (T < 16 && tid >= 64) return;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int mm = tr + 16 * i;
+    if (woffr[mm] < 0) continue;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int nn = tc + 16 * j;
+      if (woffc[nn] < 0) continue;
+      store_w(p, W + p.es * (woffr[mm] + woffc[nn]), sum[i][j]);
     }
   }
 }
@@ -692,10 +746,12 @@ void launch_skinny_ns(int sms, cudaStream_t st, const Problem& p, bool long_is_u
 }
 
 // Tile and K ranges of the tiled kernel: the least time of the busiest SM.  A K
-// block of a T x T tile takes 8 T^2 clocks of the float64 pipe, and about 1000
-// clocks more (offsets, gathers, barriers) when an SM has one tile at a time,
-// 200 when several share it.  K ranges (at least 256 columns) cost a zeroed W
-// and atomic adds: about 6000 clocks.
+// block of a T x T tile takes 8 T^2 clocks of the float64 pipe, and more for
+// offsets, gathers and barriers, the more the fewer tiles share an SM (`shared`,
+// `alone`: measured at 640 x 640 x 2000 by 2 irreps and at 64 x 64 x 16384).  K
+// ranges (2, 4, 8 or 16 of at least 256 columns) cost the exchange of their sums;
+// clusters of 8 and 16 do not spread over all SMs of a GPC (a quarter left out:
+// 64 x 64 x 16384 in 16 x 16 tiles by 8 ranges takes 279 us, not 179).
 struct TileChoice {
   int T = 64, ksplit = 1;
   int64_t kchunk = 0, units = 0;
@@ -704,13 +760,15 @@ TileChoice tile_choice(const Problem& p, int sms) {
   TileChoice best;
   double least = 0;
   for (int T : {64, 32, 16, 8}) {
+    const double shared = T == 64 ? 500 : T == 32 ? 190 : T == 16 ? 40 : 130, alone = T == 64 ? 1000 : T == 32 ? 900 : 600;
     const int64_t tiles = ((p.M + T - 1) / T) * ((p.N + T - 1) / T) * p.n_q;
-    for (int s = 1; s <= 16 && (s == 1 || p.K / s >= 256); ++s) {
+    for (int s = 1; s <= kMaxRanges && (s == 1 || p.K / s >= 256); s *= 2) {
       const int64_t blocks = ((p.K + s - 1) / s + BK - 1) / BK;   // K blocks of a range
       const int64_t ranges = (p.K + blocks * BK - 1) / (blocks * BK);
-      const int64_t units = tiles * ranges, rounds = (units + sms - 1) / sms;
-      const double time = (double)rounds * blocks * (8.0 * T * T + (units > sms ? 200 : 1000)) +
-                          (ranges > 1 ? 6000 : 0);
+      const int64_t units = tiles * ranges, at_once = ranges >= 8 ? (int64_t)sms * 3 / 4 : sms;
+      const int64_t rounds = (units + at_once - 1) / at_once;
+      double time = (double)rounds * blocks * (8.0 * T * T + (rounds > 1 ? shared : alone));
+      if (ranges > 1) time = time * (1 + 0.005 * ranges) + 3000 + 300 * ranges;
       if (best.units == 0 || time < 0.97 * least) {
         least = time;
         best.T = T;
@@ -769,20 +827,30 @@ cudaError_t launch_gemm_f64(const Problem& p, const double* u, const double* v, 
     return cudaGetLastError();
   }
   const TileChoice c = tile_choice(p, sms);
-  // (a general plan's W is zeroed as a whole before its contraction)
-  if (c.ksplit > 1 && !p.accumulate && !tables) {
-    zero_w_entries<<<sms * 4, 256, 0, st>>>(p, w);
-    ++g_kernel_launches;
-  }
   Tables t{};
   if (tables) t = *tables;
   auto kern = c.T == 64 ? gemm_f64_tiled<64> : c.T == 32 ? gemm_f64_tiled<32> : c.T == 16 ? gemm_f64_tiled<16>
                                                                                       : gemm_f64_tiled<8>;
-  const int64_t cap = (int64_t)sms * 4;
-  kern<<<(int)(c.units < cap ? c.units : cap), THREADS, 0, st>>>(
-      p, c.ksplit, c.kchunk, map_rows_fast(p.u.rows), map_rows_fast(p.v.rows), t, u, v, w);
+  if (c.units > 0x7FFFFFFF) return cudaErrorInvalidConfiguration;
+  if (c.ksplit > 8) {
+    // clusters beyond eight CTAs are opted into (every thread sets the same)
+    const cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)c.units);
+  cfg.blockDim = dim3(THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)c.ksplit;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = c.ksplit > 1 ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p, c.ksplit, c.kchunk, map_rows_fast(p.u.rows),
+                                           map_rows_fast(p.v.rows), t, u, v, w);
   ++g_kernel_launches;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace symctr

@@ -35,3 +35,25 @@ def test_tiles(sc, M, N, K, G, flip):
         a, b = (u[q].T, v[q].T) if flip else (u[q], v[q])
         want = a @ b
         assert np.all(np.abs(w[q] - want) <= 2 * (K + 2) * 2.0 ** -53 * (np.abs(a) @ np.abs(b)))
+
+
+@pytest.mark.parametrize("M,N,K,G", [(24, 24, 1500, 2), (48, 48, 1024, 3), (300, 300, 1800, 3), (200, 200, 800, 1),
+                                     (128, 128, 2048, 8), (640, 640, 2000, 2), (9, 130, 5000, 1)])
+def test_products_repeat_bit_for_bit(sc, M, N, K, G):
+    """Every tile size with K ranges (up to eight of them): the partial sums are added
+    in one order, so that a product gives the same bits each time, also where it adds
+    to W (the second products of a complex contraction)."""
+    rng = np.random.default_rng(M + K)
+    p = sc.Plan("ij,jk->ik", (G,), ((1, -1), (0,), (M, K)), ((1, -1), (0,), (K, N)), "fp64")
+    draw = lambda s: torch.from_numpy(rng.standard_normal(s)).cuda()
+    u, v = draw(p.shape_u), draw(p.shape_v)
+    uc, vc = torch.complex(u, draw(p.shape_u)), torch.complex(v, draw(p.shape_v))
+    first, firstc = p.contract(u, v), p.contract_complex(uc, vc)
+    for _ in range(20):
+        assert torch.equal(p.contract(u, v), first)
+        assert torch.equal(p.contract_complex(uc, vc), firstc)
+    bound = 2 * (K + 2) * 2.0 ** -53 * (u.abs() @ v.abs()).reshape(first.shape)
+    assert bool(((first - (u @ v).reshape(first.shape)).abs() <= bound).all())
+    want = uc @ vc
+    bound = 4 * (K + 2) * 2.0 ** -53 * (uc.abs() @ vc.abs()).reshape(firstc.shape)
+    assert bool(((firstc - want.reshape(firstc.shape)).abs() <= bound).all())
