@@ -259,25 +259,10 @@ def prep_bytes(pl):
     elems = i.aligned_numel_u + i.aligned_numel_v
     if i.precision == 1:
         return elems * (8 + 2 * digit_planes(i.n_slices)) + 4 * i.n_q * (i.M + i.N)
-    direct = tf32_direct(pl)
+    direct = pl.gemm_kernel()[1]
     if direct is not None:
         elems = (i.aligned_numel_v, i.aligned_numel_u)[direct]
     return elems * (8 + 4)
-
-
-def tf32_direct(pl):
-    """The operand (0 or 1) whose float64 entries the TF32 GEMM reads itself, or
-    None: the shape rule of tf32_direct_operand in transforms.cu (one pass, real,
-    uniform plans)."""
-    i = pl.info
-    inputs = pl.einsum.replace(" ", "").split("->")[0].split(",")
-    for op in (0, 1):
-        rows, other = ((i.M, i.N), (i.N, i.M))[op]
-        last, dim = inputs[op][-1], (pl.sym_u, pl.sym_v)[op].dims[-1]
-        if other <= 512 and rows >= 4 * other and (rows + 127) // 128 * i.n_q >= 128 and i.K >= 64 \
-                and last in inputs[1 - op] and dim % 2 == 0:
-            return op
-    return None
 
 
 def prep_kernels(pl):
@@ -307,21 +292,20 @@ def rooflines(args, plans, prep, gemm, pk):
     its launches in one step / their CUDA-event time in that step."""
     out = []
     gemm_ms = sum(gemm)
+    kernel = plans[0].gemm_kernel()[0]
     if args.precision == "split_bf16":
         planes = [digit_planes(pl.info.n_slices) for pl in plans]
         pairs = [n * (n + 1) // 2 for n in planes]
         work = sum(pl.useful_flops * k for pl, k in zip(plans, pairs))
-        kernel = "gemm_tc10_kernel" if plans[0].info.n_slices == 5 else "gemm_tc_kernel"
         bound, unit, peak = "tensor", "TFLOP/s", pk["bf16_tflops"]
         peak_src = f"{pk['src']} bf16 burst"
     elif args.precision == "tf32":
         work = sum(pl.useful_flops for pl in plans)
-        kernel = "gemm_tc_kernel" if tf32_direct(plans[0]) is None else "gemm_tf32_direct_kernel"
         bound, unit, peak = "tensor", "TFLOP/s", pk["bf16_tflops"] / 2
         peak_src = f"{pk['src']} bf16 burst x 1/2 (nominal tf32:bf16 ratio)"
     else:
         work = sum(pl.useful_flops for pl in plans)
-        kernel, bound, unit, peak = "gemm_f64", "alu", "TFLOP/s", 1.25
+        bound, unit, peak = "alu", "TFLOP/s", 1.25
         peak_src = "1.25 TFLOP/s nominal FP64 (152 SMs x FP64 units x clock; cuBLAS DGEMM measured 1.1)"
     achieved = work / (gemm_ms * 1e-3) / 1e12
     key = f"{kernel}/{args.precision}/{args.workload}"

@@ -245,6 +245,13 @@ SYMCTR_API symctr_status symctr_plan_chain(symctr_plan* plan, const symctr_plan*
 /* Fill *out with the plan's derived quantities.  Host only. */
 SYMCTR_API symctr_status symctr_plan_query(const symctr_plan* plan, symctr_plan_info* out);
 
+/* Name of the kernel that runs the plan's GEMM in symctr_contract (one pass, 16-byte
+ * aligned tensors): "gemm_tc10_kernel" (default split form), "gemm_tc_kernel",
+ * "gemm_tf32_direct_kernel" or "gemm_f64".  direct_operand (may be NULL) receives
+ * the operand (0 = U, 1 = V) whose float64 entries that kernel reads itself,
+ * without a prepared copy, or -1.  "" for NULL or a plan without work.  Host only. */
+SYMCTR_API const char* symctr_plan_gemm_kernel(const symctr_plan* plan, int* direct_operand);
+
 /* Give the plan a device-resident copy of its offset tables (the row and column
  * offsets of Alg. 2's aligned operands in the standard reduced forms, computed
  * on the host at plan creation, including those of the backward's two

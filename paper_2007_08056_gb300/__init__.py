@@ -124,6 +124,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
                                             ctypes.c_size_t, P]
     lib.symctr_plan_workspace_bytes_complex.argtypes = [P]
     lib.symctr_plan_workspace_bytes_complex.restype = ctypes.c_uint64
+    lib.symctr_plan_gemm_kernel.argtypes = [P, ctypes.POINTER(ctypes.c_int)]
+    lib.symctr_plan_gemm_kernel.restype = ctypes.c_char_p
     lib.symctr_plan_attach_tables.argtypes = [P, P, ctypes.c_size_t, P]
     lib.symctr_plan_chain.argtypes = [P, P, P, ctypes.c_int]
     lib.symctr_plan_destroy.argtypes = [P]
@@ -508,6 +510,13 @@ class Plan:
         _check(load().symctr_profile_read(self._h, ctypes.byref(a), ctypes.byref(b),
                                           ctypes.byref(n)))
         return a.value, b.value, n.value
+
+    def gemm_kernel(self):
+        """(name of the kernel that runs the plan's GEMM, the operand whose float64
+        entries it reads itself or None): symctr_plan_gemm_kernel."""
+        op = ctypes.c_int()
+        name = load().symctr_plan_gemm_kernel(self._h, ctypes.byref(op)).decode()
+        return name, None if op.value < 0 else op.value
 
     @property
     def useful_flops(self) -> float:

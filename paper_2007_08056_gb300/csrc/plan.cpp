@@ -1417,6 +1417,16 @@ uint64_t symctr_plan_workspace_bytes_complex(const symctr_plan* P) {
   return complex_layout(P, UINT64_MAX, &both, &acc_n) ? both.bytes : P->ws_bytes;
 }
 
+const char* symctr_plan_gemm_kernel(const symctr_plan* P, int* direct_operand) {
+  if (direct_operand) *direct_operand = -1;
+  if (!P || P->run.n_q < 1) return "";
+  if (!P->tensor_core) return "gemm_f64";
+  if (P->prec == SYMCTR_SPLIT_BF16) return P->n_slices == 5 ? "gemm_tc10_kernel" : "gemm_tc_kernel";
+  const int op = tf32_direct_operand(P->run, nullptr, nullptr);   // (any aligned address)
+  if (direct_operand) *direct_operand = op;
+  return op >= 0 ? "gemm_tf32_direct_kernel" : "gemm_tc_kernel";
+}
+
 symctr_status symctr_plan_query(const symctr_plan* P, symctr_plan_info* o) {
   if (!P || !o) return fail(SYMCTR_ERR_NULLPTR, "NULL argument");
   std::memset(o, 0, sizeof(*o));

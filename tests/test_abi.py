@@ -158,6 +158,24 @@ def test_workspace_of_complex_contractions():
     assert g.info.workspace_bytes < need < 2 * g.info.workspace_bytes + 16 * g.info.n_q * g.info.M * g.info.N
 
 
+def test_gemm_kernel_of_a_plan_is_reported():
+    pp, cc = WL.PP, WL.CC_LADDER
+    ladder = lambda prec, c=32, slices=0: sc.Plan(cc.einsum, (8,), (pp, (0,), (32, 32, 32, c)),
+                                                  (pp, (0,), (32, c, 8, 8)), prec, n_slices=slices)
+    assert ladder("split_bf16").gemm_kernel() == ("gemm_tc10_kernel", None)
+    assert ladder("split_bf16", slices=4).gemm_kernel() == ("gemm_tc_kernel", None)
+    assert ladder("tf32").gemm_kernel() == ("gemm_tf32_direct_kernel", 0)
+    assert ladder("tf32", c=31).gemm_kernel() == ("gemm_tc_kernel", None)     # pairs of columns split
+    assert ladder("fp64").gemm_kernel() == ("gemm_f64", None)
+    # the other operand long: both have the contracted modes last
+    v = sc.Plan("xyk,abk->abxy", (8,), ((1, 1, -1), (0,), (8, 8, 64)), ((1, 1, -1), (0,), (64, 64, 64)), "tf32")
+    assert v.gemm_kernel() == ("gemm_tf32_direct_kernel", 1)
+    y = sc.Plan(WL.PEPS_Y, WL.PEPS_MODULI, (WL.PEPS_T.signs, (0, 0), WL.PEPS_T.dims),
+                (WL.PEPS_ENV.signs, (0, 0), WL.PEPS_ENV.dims), "split_bf16")
+    assert y.gemm_kernel() == ("gemm_f64", None)
+    assert sc.load().symctr_plan_gemm_kernel(None, None) == b""
+
+
 def test_workspace_too_small_is_rejected_before_any_launch():
     """The size check happens on the host, so it needs no GPU."""
     p = sc.Plan(WL.Z3_ORDER4.einsum, (3,), (WL.PP, (0,), (4,) * 4), (WL.PP, (0,), (4,) * 4),
