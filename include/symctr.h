@@ -88,8 +88,9 @@ typedef enum {
 
 typedef enum {
   SYMCTR_FP64 = 0,        /* float64 FMA throughout */
-  SYMCTR_SPLIT_BF16 = 1,  /* Ozaki-style BF16 slices on tcgen05, exact FP32 partial
-                             sums, integer recombination, one rounding to float64 */
+  SYMCTR_SPLIT_BF16 = 1,  /* Ozaki-style 16-bit digits (FP16; BF16 for n_slices other than
+                             5) on tcgen05, exact FP32 sums of the leading products,
+                             integer recombination, one rounding to float64 */
   SYMCTR_TF32 = 2         /* operands rounded to TF32 on tcgen05, FP32 accumulation */
 } symctr_precision;
 

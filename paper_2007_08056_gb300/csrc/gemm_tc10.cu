@@ -52,7 +52,8 @@
 // D = 23 1.02 -> 0.81 ms, 40960 x 640 x 640 by 10 irreps 5.11 -> 3.59 ms (3.99
 // with a CTA to a tile and the longer writes, 3.70 with those alone).
 // The drain loop leaves no register to spare: with 80 bytes of spills instead of
-// 32 that last case takes 4.01 ms.
+// 32 that last case takes 4.01 ms (the 128 x 64 tile, at 80 registers a thread for
+// two CTAs, spills 108).
 // Every wait is bounded (see tc_common.cuh).
 #include "tc_common.cuh"
 

@@ -103,16 +103,19 @@ __global__ void __launch_bounds__(THREADS) align_kernel(Problem p, OperandMap m,
 }
 
 // ---------------------------------------------------------------------------
-// Split-BF16 operand preparation (Ozaki-style splitting, integer arithmetic
-// only: GB300 has very little float64 throughput).
+// Operand preparation of the split form (Ozaki-style splitting, integer
+// arithmetic only: GB300 has very little float64 throughput).
 //
-// For aligned row r with largest binary exponent E_r (|x| < 2^(E_r+1)), each
-// entry is written as y = x / 2^(E_r+1) in (-1, 1) and rounded to the integer
-// X = round(y * 2^(8S-1)), |X| <= 2^(8S-1).  X is cut into S balanced base-256
-// digits a_0..a_{S-1} with a_i in [-128, 128], so y ~= sum_i a_i 2^(-7-8i) with
-// error <= 2^(-8S).  Slice i stores a_i * 2^(-8i) as BF16 (exact: a_i has at
-// most 8 significant bits), so that every slice-pair product lands at its own
-// scale 2^(-8(i+j)) and |a_i b_j| <= 2^14.
+// For aligned row r with binary exponent E_r (|x| < 2^(E_r+1), row_exponent),
+// each entry is written as y = x / 2^(E_r+1) in (-1, 1) and rounded to the
+// integer X = round(y * 2^(8S-1)), |X| <= 2^(8S-1), which is cut into planes of
+// 16-bit digits (P = digit_planes(S) of them):
+//   S = 5 (default)  four balanced base-1024 digits as FP16 integers (below);
+//   other S          S balanced base-256 digits a_0..a_{S-1} in [-128, 128], so
+//     y ~= sum_i a_i 2^(-7-8i) with error <= 2^(-8S).  Slice i stores
+//     a_i * 2^(-8i) as BF16 (exact: a_i has at most 8 significant bits), so that
+//     every slice-pair product lands at its own scale 2^(-8(i+j)) and
+//     |a_i b_j| <= 2^14.
 // ---------------------------------------------------------------------------
 
 // Row exponents, stored biased: E + kExpBias for a row whose largest entry
@@ -177,7 +180,7 @@ __device__ __forceinline__ int row_k0(int32_t key, int S) {
   return key == 0 ? 4096 : key - kExpBias + 1077 - 8 * S;
 }
 
-// Balanced base-256 digits by byte extraction: with B = 0x80 * (256^S - 1)/255,
+// Balanced base-256 digits (S other than 5) by byte extraction: with B = 0x80 * (256^S - 1)/255,
 // Y = X + B has bytes (a_k + 128) for the low S-1 digits and (a_top + 128) in
 // [0, 256] above them (no carries: every shifted digit lies in [0, 255]).
 __host__ __device__ constexpr uint64_t digit_bias(int S) {
@@ -377,8 +380,8 @@ __device__ void scan_tile(const PrepArgs& a, int op, uint32_t tile, int64_t* rof
   }
 }
 
-// Writes the S slices of two adjacent columns (c, c+1) of one row: one
-// packed BF16 pair per slice (the conversion is exact, every digit value has
+// Writes the S slices of two adjacent columns (c, c+1) of one row (S other than
+// 5): one packed BF16 pair per slice (the conversion is exact, every digit value has
 // at most 8 significant bits).
 template <int S, int I = 0>
 __device__ __forceinline__ void put_digits(uint64_t y0, uint64_t y1, uint32_t* dst, int64_t stride) {
@@ -444,7 +447,7 @@ __device__ __forceinline__ void put_slices_pair(double x0, double x1, int k0, ui
   }
 }
 
-// Four adjacent columns of one row: per slice, four BF16 digits in one 8-byte
+// Four adjacent columns of one row: per slice, four digits in one 8-byte
 // store (dst and stride in units of uint2).
 template <int S, int I = 0>
 __device__ __forceinline__ void put_digits_quad(const uint64_t (&y)[4], uint2* dst, int64_t stride) {
@@ -500,7 +503,7 @@ __device__ __forceinline__ void put_pair(const PrepArgs& a, int op, double x0, d
 }
 
 // One work unit of the padded aligned operand: 32 rows by SLICE_GROUP x 64
-// columns (S slices; S = 0: the TF32 copy).  Column-contiguous operands are
+// columns (the digit planes; S = 0: the TF32 copy).  Column-contiguous operands are
 // read along the columns straight from global memory (16-byte loads when every
 // offset is even), row-contiguous ones go through shared memory, 64 columns at
 // a time, so that both the gather and the slice stores are coalesced.  The row
@@ -658,7 +661,7 @@ __device__ void slice_unit(const PrepArgs& a, int op, uint32_t unit, int64_t* ro
 // offset tables are already in the workspace):
 //   phase 1  zeroed split-K accumulators and (split form) the per-row
 //            exponent maxima of U and V;
-//   phase 2  BF16 slices (split) or TF32 copies of U and V.
+//   phase 2  digit planes (split) or TF32 copies of U and V.
 template <int S>
 __global__ void __launch_bounds__(THREADS, 4) prep_kernel(PrepArgs a) {
   __shared__ int64_t roff[TILE], coff[kScanWidth];
@@ -722,7 +725,7 @@ struct RowStreamArgs {
   const int64_t* rtab;      // [n_q][R] row offsets
   const int64_t* ctab;      // [n_q][K] column offsets (run starts read at multiples of L)
   const double* src;
-  uint32_t* dst;            // BF16 digit pairs: [S][n_q][R][kpad / 2]
+  uint32_t* dst;            // digit pairs: [P][n_q][R][kpad / 2]
   int64_t slice_stride;     // n_q * R * kpad (elements)
   int32_t* exps;            // [n_q][R] biased row exponents
   unsigned* err;
@@ -1180,7 +1183,7 @@ struct RowTileArgs {
   int rlog;                  // rows per CTA = 2^rlog
   uint32_t units[2];         // (irrep, row block) units of U and of V (0: not prepared here)
   const double* src[2];
-  uint32_t* dst[2];          // BF16 digit pairs: [S][n_q][R][kpad / 2]
+  uint32_t* dst[2];          // digit pairs: [P][n_q][R][kpad / 2]
   int32_t* exps[2];          // [n_q][R] biased row exponents
   bool fast_rows[2];
   bool pair_ok[2];           // column-contiguous with every offset of an even column even

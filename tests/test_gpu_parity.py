@@ -2,7 +2,7 @@
 
 Tolerances (relative Frobenius error against the oracle's block loop):
   fp64        <= 1e-12   (float64 FMA; summation order differs)
-  split_bf16  <= 1e-10   (5 BF16 slices of 8 bits: truncation ~2^-39 per
+  split_bf16  <= 1e-10   (four FP16 digits of 10 bits: truncation ~2^-39 per
                           operand entry relative to its row maximum)
   tf32        <= 1e-2    (operands rounded to 11 significant bits)
 Alignment transforms are compared bit for bit.
@@ -237,8 +237,8 @@ def test_ragged_tiles(sc, precision):
 
 @pytest.mark.parametrize("k_blocks", [1, 3, 64, 257])
 def test_split_exactness_all_positive(sc, k_blocks):
-    """All-positive data makes every slice-pair partial sum grow linearly with K:
-    without exact flushes of the top diagonals the FP32 accumulators would
+    """All-positive data makes the sums of the leading digits' products grow linearly
+    with K: without exact drains of the top diagonals the FP32 accumulators would
     round.  K up to 8224 (257 stages of 32)."""
     G, Dm, Dn = 2, 130, 70
     Dk = 32 * k_blocks
@@ -354,11 +354,12 @@ def test_no_irrep_carries_work(sc, precision):
 
 @pytest.mark.parametrize("k_sectors,D", [(2, 64), (2, 4096), (4, 8192)])
 def test_split_bit_exact_on_integer_inputs(sc, k_sectors, D):
-    """Integer entries with |x| <= 2^12 are exactly two balanced BF16 digits
-    at their row scale, so every slice-pair product lands in the exact
-    diagonals 0..2: the split form must return the exact integer matrix
-    product rounded once to float64, bit for bit.  Rows at the maximum
-    magnitude (all digits at the bound) drive every drain to its limit."""
+    """Integer entries with |x| <= 2^12 are exactly two FP16 digits at their row
+    scale, x / 16 rounded and a multiple of 64: their products lie in the exact
+    diagonals 0 and 1 and, as multiples of 2^12 that FP32 sums exactly, in diagonal
+    2, so the split form must return the exact integer matrix product rounded once
+    to float64, bit for bit.  Rows of the largest magnitude have the leading digit
+    256; leading digits at their limit are in test_gpu_split_digits.py."""
     G = k_sectors
     su = ((1, -1), (0,), (128, D))
     sv = ((1, -1), (0,), (D, 96))
@@ -387,7 +388,7 @@ def test_single_read_prep_bit_exact_on_integer_inputs(sc, einsum, D_i, D_j, prep
     rows streamed by bulk copies of contiguous runs, by one CTA up to K = 8192
     and by clusters of 2 to 8 CTAs holding one segment each beyond; 2/3: whole
     short rows per CTA, gathered along the rows or across them; neither: the
-    two-phase kernel), alone and side by side: integer inputs of two BF16 digits must give
+    two-phase kernel), alone and side by side: integer inputs of two FP16 digits must give
     the exact integer product rounded once, bit for bit."""
     G, D_k = 2, 72
     su = ((1, -1), (0,), (D_i, D_j))
@@ -401,8 +402,8 @@ def test_single_read_prep_bit_exact_on_integer_inputs(sc, einsum, D_i, D_j, prep
     # a row of subnormals k * 2^-1050, |k| <= 127: every high word is zero (the
     # row scale comes from the exact pass over the whole bit patterns) and the
     # row scale is the clamped one, 2^(8S - 1076) = 2^-1036 at S = 5, at which
-    # each entry is the single BF16 digit k * 2^-8 below the top: its products
-    # with V's two digits stay in the exact diagonals
+    # each entry is the single digit 16 k below the top one: its products with V's
+    # two digits stay in diagonals 1 and 2, which hold them exactly
     ks = rng.integers(-127, 128, size=(G, D_j))
     u[:, 7, :] = np.ldexp(ks.astype(np.float64), -1050)
     p = sc.Plan(einsum, (G,), su, sv, "split_bf16")

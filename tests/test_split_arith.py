@@ -1,15 +1,17 @@
-"""Host checks of the FP32 identities the split-BF16 GEMM's epilogue relies on
-(no GPU): FP32 arithmetic is emulated with numpy float32, whose operations
-round to nearest even like the kernel's.
+"""Host checks of the arithmetic that the split GEMMs rely on (no GPU).  The FP32
+identities of the epilogue for n_slices 2, 3, 4 and 6 (BF16 digits), emulated with
+numpy float32, whose operations round to nearest even like the kernel's:
 
 * Magic-number rounding: for |y| <= 2^22, float32(y + 1.5 * 2^23) has the
   integer round(y) (ties to even) in its low mantissa bits.
 * The final drain's round(acc3 * 2^24) for |acc3| < 64: h = round(acc3 * 2^16)
   by the magic number, the remainder acc3 - h 2^-16 exact in FP32, and
   round(acc3 * 2^24) = 2^8 h + round(remainder * 2^24).
-* The default split's row scale and digits (tests/native, compiled with the host
-  compiler against the library's internal header): no leading digit above 511, and
-  the sums between two drains below 2^24."""
+The default split (FP16 digits):
+
+* The row scale and digits (tests/native, compiled with the host compiler against
+  the library's internal header): no leading digit above 511, and the sums between
+  two drains below 2^24."""
 import os
 import shutil
 import subprocess
@@ -61,7 +63,7 @@ def test_acc3_rounding_matches_float64():
 
 
 def test_drain_bound_fits_the_magic_window():
-    """A drain carries at most 3 x 64, 2 x 128 or 1 x 256 slice products of
+    """BF16 digits: a drain carries at most 3 x 64, 2 x 128 or 1 x 256 products of
     |a_i b_j| <= 2^14 (diagonals 2, 1, 0), so the FP32 sum is an integer
     within the magic-number window 2^22."""
     assert max(3 * 64, 2 * 128, 1 * 256) * 2 ** 14 <= 2 ** 22
