@@ -339,9 +339,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tma_load_4d(&tma_b, &full[st], sb, kc, (int)n0, b);
         ++issued;
       }
-      // the last copies land before the CTA exits
-      for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-        wait_landed(&full[kb % STAGES], (kb / STAGES) & 1, ctl);
+      ctl->copies = (uint32_t)issued;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -390,7 +388,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
       tc_commit(acc_full);
       tc_commit(drain);
-      wait_landed(drain, 0, ctl);
+      wait_phase(drain, 0, ctl, kTimeoutCycles / 2);
     }
   } else if (warp >= EPI_WARP0) {
     // ------------------------------------------------------------ epilogue
@@ -608,6 +606,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // a split-K rounding kernel behind this one may start its launch now
   asm volatile("griddepcontrol.launch_dependents;");
   __syncthreads();
+  if (ctl->abort) {
+    land(full, STAGES, drain, ctl);
+    __syncthreads();
+  }
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();

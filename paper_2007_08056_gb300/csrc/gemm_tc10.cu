@@ -203,6 +203,21 @@ __device__ __forceinline__ bool all_ok(bool ok) {
   return r != 0;
 }
 
+// After an abort, before the CTA gives its memory back (out of line: see wait_landed):
+// thread i < STAGES waits for the last copy into stage i, the issuing threads for
+// their MMAs.
+template <int H>
+__device__ __noinline__ void land10(uint64_t* full, uint64_t* issued, Ctl* ctl) {
+  const int t = threadIdx.x, h = t / 32 - 1;
+  uint64_t* bar = nullptr;
+  if (t < Cfg<H>::STAGES && ((ctl->copies >> t) & 1)) bar = &full[t];
+  if (t % 32 == 0 && h >= 0 && h < H) {
+    bar = &issued[h];
+    tc_commit(bar);
+  }
+  if (bar) wait_landed(bar, t < Cfg<H>::STAGES ? ((ctl->phases >> t) & 1) ^ 1 : 0, ctl);
+}
+
 template <int H, bool GEN>
 __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
     gemm_tc10_kernel(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b,
@@ -221,7 +236,7 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
   uint64_t* acc_full = drained + 2;      // a tile's MMAs are done
   uint64_t* zero_done = acc_full + 1;    // its accumulators are read out and zeroed
   uint64_t* staged = zero_done + 1;      // its results have left the staging
-  uint64_t* issued = staged + 1;         // [2] all of an issuing thread's MMAs are done
+  uint64_t* issued = staged + 1;         // [2] after an abort: all of an issuing thread's MMAs are done
   uint8_t* tabs = (uint8_t*)(issued + 2);      // [2] tables of this tile and the last one
   uint32_t* tmem_slot = (uint32_t*)(tabs + 2 * C::TAB);
   Ctl* ctl = (Ctl*)(tmem_slot + 4);
@@ -316,9 +331,8 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
           st = st + 1 == STAGES ? 0 : st + 1;
         }
       }
-      // the last copies land before the CTA exits
-      for (int s = 0; s < STAGES; ++s)
-        if ((live >> s) & 1) wait_landed(&full[s], ((ph >> s) & 1) ^ 1, ctl);
+      ctl->copies = live;
+      ctl->phases = ph;
     }
   } else if (warp <= H) {
     // ------------------------------------------------------------ MMA issuers
@@ -369,9 +383,6 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
         }
         tc_commit(acc_full);
       }
-      // the last MMAs are done before the CTA gives its TMEM back, after an abort too
-      tc_commit(&issued[h]);
-      wait_landed(&issued[h], 0, ctl);
     }
   } else if (warp >= EPI_WARP0) {
     // ------------------------------------------------------------ epilogue
@@ -619,6 +630,10 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
   // a split-K rounding kernel behind this one may start its launch now
   asm volatile("griddepcontrol.launch_dependents;");
   __syncthreads();
+  if (ctl->abort) {
+    land10<H>(full, issued, ctl);
+    __syncthreads();
+  }
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();

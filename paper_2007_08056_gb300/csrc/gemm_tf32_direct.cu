@@ -173,9 +173,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         for (int i = 0; i < NB; ++i) tma_load_4d(&tma_b, &b_full[st], sb + i * B_BYTES, kb * KST, i * BH, b);
         ++issued;
       }
-      // the last copies land before the CTA exits
-      for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-        wait_landed(&b_full[kb % STAGES], (kb / STAGES) & 1, ctl);
+      ctl->copies = (uint32_t)issued;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -204,7 +202,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tc_commit(&empty[st]);
       }
       tc_commit(acc_full);
-      wait_landed(acc_full, 0, ctl);
+      wait_phase(acc_full, 0, ctl, kTimeoutCycles / 2);
     }
   } else if (warp >= W0) {
     // ------------------------------------------------------------ long operand
@@ -336,6 +334,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     tc_fence_before();
   }
   __syncthreads();
+  if (ctl->abort) {
+    land(b_full, STAGES, acc_full, ctl);
+    __syncthreads();
+  }
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();

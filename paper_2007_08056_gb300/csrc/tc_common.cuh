@@ -44,6 +44,9 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 struct Ctl {
   volatile int abort;
   unsigned* err;
+  // the producer's copies, for the waits after an abort: how many, or (gemm_tc10.cu)
+  // the stages used and the parities of their next use
+  uint32_t copies, phases;
 };
 
 // Bounded wait: true when the phase completed; false on timeout or abort.
@@ -92,11 +95,15 @@ __device__ __forceinline__ bool wait_phase_sleep(uint64_t* bar, uint32_t parity,
   }
 }
 
-// Before a CTA leaves: wait for its own copies or MMAs in flight, after an abort
-// too (the waits above give up at once then), so that none writes to shared
-// memory or TMEM that the next CTA holds.  Bounded by the limit alone.
-__device__ __forceinline__ bool wait_landed(uint64_t* bar, uint32_t parity, Ctl* ctl,
-                                            long long limit = kTimeoutCycles / 2) {
+// Before a CTA leaves after an abort: wait for its own copies or MMAs in flight
+// (the waits above give up at once then), so that none writes to shared memory or
+// TMEM that the next CTA holds.  Bounded by the limit alone.  The kernels do so
+// behind their last barrier, when no thread can set the abort flag any more and
+// all see the same; without an abort everything in flight has been consumed.  Out
+// of line: within the kernels this code, though never run, cost the ladder in TF32
+// 0.5% and the split GEMM 1.2% (40960 x 640 x 640 by 10 irreps).
+static __device__ __noinline__ bool wait_landed(uint64_t* bar, uint32_t parity, Ctl* ctl,
+                                                long long limit = kTimeoutCycles / 2) {
   const long long t0 = clock64();
   while (!mbar_test_sleep(bar, parity)) {
     if (clock64() - t0 > limit) {
@@ -106,6 +113,14 @@ __device__ __forceinline__ bool wait_landed(uint64_t* bar, uint32_t parity, Ctl*
     }
   }
   return true;
+}
+
+// The same for a kernel whose producer made ctl->copies copies round the stages'
+// barriers `full` and whose issuing thread (32) committed its MMAs to `mmas`.
+__device__ __forceinline__ void land(uint64_t* full, int stages, uint64_t* mmas, Ctl* ctl) {
+  const int i = threadIdx.x, last = (int)ctl->copies - 1 - i;   // thread i < stages: one of the last copies
+  uint64_t* bar = i < stages && last >= 0 ? &full[last % stages] : i == 32 ? mmas : nullptr;
+  if (bar) wait_landed(bar, i < stages ? (last / stages) & 1 : 0, ctl);
 }
 
 // Box of a [planes][batches][rows][k] map at (k = c0, row = c1, batch = c2, plane 0).
