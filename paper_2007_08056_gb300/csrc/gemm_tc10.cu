@@ -391,7 +391,6 @@ __global__ void __launch_bounds__(Cfg<H>::NTHREADS, 3 - H)
     const int ew = warp - EPI_WARP0;      // 0..15
     const int quad = warp & 3;            // TMEM lane quadrant this warp may access
     const int h = ew >> 3, part = (ew >> 2) & 1;   // half of the tile, half of its columns
-    const int row = quad * 32 + lane;
     // accumulator of diagonal d: lane_base + 64 d
     const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(4 * HN * h + part * 32);
     // Running sums in units 8 (s0) and 8 x 2^-10 (s1): a drain moves the
