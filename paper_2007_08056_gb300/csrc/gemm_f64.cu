@@ -43,8 +43,8 @@ __host__ __device__ inline bool map_rows_fast(const AxisMap& rows) {
 // all of them (tile_choice): 48 x 48 x 48 by 3 irreps ran on three SMs with
 // 64 x 64 tiles, 65 -> 17 us (launch-bound) with 8 x 8; the two MPS contractions
 // 128 x 2048 x 128 and 128 x 128 x 2048 by 8 irreps, on 3.4 such tiles per SM and
-// on 128 of 152 SMs, 1177 -> 922 us with 16 x 16 (909 us at the float64 rate of a
-// large product).  Column offsets are computed for kKc columns of K at a time,
+// on 128 of 152 SMs, 1177 -> 922 us with 16 x 16 (866 us at the float64 rate of the
+// CC ladder, 443 ms, 0.99 of the pipe; 471 ms before).  Column offsets are computed for kKc columns of K at a time,
 // one per thread; the next K block's gathers are in flight while this one is
 // multiplied.  One CTA to a tile and range: a grid of four CTAs per SM walking
 // them left SMs with one more or less than their share (640 x 640 x 2000 by 2
