@@ -38,9 +38,10 @@ def test_tiles(sc, M, N, K, G, flip):
 
 
 @pytest.mark.parametrize("M,N,K,G", [(24, 24, 1500, 2), (48, 48, 1024, 3), (300, 300, 1800, 3), (200, 200, 800, 1),
-                                     (128, 128, 2048, 8), (640, 640, 2000, 2), (9, 130, 5000, 1)])
+                                     (128, 128, 2048, 8), (640, 640, 2000, 2), (9, 130, 5000, 1),
+                                     (32, 32, 4096, 1)])
 def test_products_repeat_bit_for_bit(sc, M, N, K, G):
-    """Every tile size with K ranges (up to eight of them): the partial sums are added
+    """Every tile size with K ranges (2 to 16 of them): the partial sums are added
     in one order, so that a product gives the same bits each time, also where it adds
     to W (the second products of a complex contraction)."""
     rng = np.random.default_rng(M + K)

@@ -179,3 +179,25 @@ def test_general_dropped_rows_on_every_route(sc, precision):
             assert rel(w.cpu().numpy(), want) <= TOL[precision]
         plan.check_device_error()
         plan.check_device_error(ws)
+
+
+def test_general_float64_k_ranges(sc):
+    """The float64 form with K ranges read through the tables (few rows and columns,
+    a contracted pair of 2 and 4 sectors in ragged blocks): parity, exact zeros, and
+    the same bits each time, real and complex."""
+    rng = np.random.default_rng(6200)
+    ragged = lambda h, d: tuple(int(x) for x in rng.integers(d // 2, d + 1, h))
+    sk, sl, sa, sc_ = ragged(2, 50), ragged(4, 60), ragged(4, 20), ragged(2, 24)
+    su = O.Sym((1, 1, -1), (0,), (20, 50, 60), (4, 2, 4), (sa, sk, sl))
+    sv = O.Sym((-1, 1, 1), (2,), (50, 60, 24), (2, 4, 2), (sk, sl, sc_))
+    g = O.Group((4,))
+    p = O.plan("akl,klc->ac", g, su, sv)
+    u, v = (O.sanitize(g, t, rng.standard_normal(O.reduced_shape(g, t))) for t in (su, sv))
+    plan = check(sc, p, u, v, "fp64", rng)
+    assert plan.info.K >= 2048
+    ud, vd = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+    uc, vc = torch.complex(ud, ud.flip(-1)), torch.complex(vd, vd.flip(-1))
+    w, wc = plan.contract(ud, vd), plan.contract_complex(uc, vc)
+    for _ in range(10):
+        assert torch.equal(plan.contract(ud, vd), w)
+        assert torch.equal(plan.contract_complex(uc, vc), wc)
