@@ -289,7 +289,10 @@ SYMCTR_API symctr_status symctr_align(const symctr_plan* plan, int operand, int 
  *  workspace : device scratch (256-byte aligned) of at least workspace_bytes_min bytes;
  *              with less than workspace_bytes the irreps Q are processed in several
  *              passes, each holding the aligned operands of as many irreps as fit.  Its
- *              first word receives device-side error codes. */
+ *              first word receives device-side error codes.
+ * The same call gives the same bits each time, but for products of the float64
+ * kernels with an aligned side of at most 8 rows and a long K, whose K ranges add
+ * up in no fixed order. */
 SYMCTR_API symctr_status symctr_contract(const symctr_plan* plan, const double* u_red, const double* v_red,
                               double* w_red, void* workspace, size_t workspace_bytes,
                               void* stream);
